@@ -16,27 +16,25 @@
 // and every tile with a short list with one CTA, one warp per block
 // (described at the kernel).
 //
-// The one-pass kernel of statistics frames, the split passes and the
-// chunked passes of training frames below take one CTA per tile (or chunk of
-// its list), one thread per pixel, each warp an 8x4 block of the tile.  A CTA walks depth-ordered pairs in batches of 256, software
-// pipelined:
-// while the warps composite batch k from one half of a shared double buffer,
-// each thread holds in registers the record it loaded for batch k+1; after
-// compositing it stages that record into the other half (with the warp
-// blocks its reach box overlaps as an 8-bit mask, and the exponent
-// pre-scaled to base 2: e^q = 2^(q log2 e) on the hardware ex2 unit) and
-// issues the loads of batch k+2.  Each warp walks only the splats marked for
-// its block; the CTA leaves once every pixel is saturated.
+// Statistics and training frames take k_blend_walk: a CTA per tile, a warp
+// per 8x4 block of it, one pixel per lane, each warp walking its block's
+// pairs on its own.  So do the split passes of long lists: a list is split
+// in depth order (the compositing operator is associative); the first
+// `budget` pairs of every tile are composited as above (kBudget in plain
+// frames, kTrainBudget in training), tiles with unsaturated pixels left hand
+// the rest to k_blend_chunks, which composites chunks of kChunk pairs in
+// parallel, each from T = 1 and only for pixels still open; k_blend_merge
+// then combines, per pixel, C += T C_k, T *= T_k in order, up to the chunk
+// (if any) inside which the pixel meets the stop rule (T T_k < 1e-4);
+// k_blend_fix composites each such chunk again, in parallel over chunks, for
+// its stopping pixels from their true T, so the stop rule holds exactly as in
+// the definition.
 //
-// Long lists are split in depth order (the compositing operator is
-// associative): pass 1 composites the first kBudget pairs of every tile;
-// tiles with unsaturated pixels left hand the rest to pass 2, which
-// composites chunks of kChunk pairs in parallel, each from T = 1 and only
-// for pixels pass 1 left open; the merge pass then combines, per pixel,
-// C += T C_k, T *= T_k in order, up to the chunk (if any) inside which the
-// pixel meets the stop rule (T T_k < 1e-4); the fix-up pass composites each
-// such chunk again, in parallel over chunks, for its stopping pixels from
-// their true T, so the stop rule holds exactly as in the definition.
+// Rounding of T.  The stop rule compares T with a constant, so an ulp of T
+// can decide whether a pixel takes one more splat (up to 1e-3 in colour).  T
+// is therefore always the product over the same groups of pairs: in training
+// frames over chunks of kChunk pairs whether they are composited in turn
+// (the walk, settle_group) or in parallel.
 #include <algorithm>
 
 #include "crowdsplat.h"
@@ -47,10 +45,15 @@ namespace cs {
 constexpr int kBlendThreads = kTile * kTile;
 constexpr int kBlockW = kBlendBlockW, kBlockH = kBlendBlockH;  // pixels per warp
 constexpr float kLog2e = 1.4426950408889634f;
-constexpr uint32_t kBudget = kBlendBudget;  // pairs of pass 1 per tile
+constexpr uint32_t kBudget = kBlendBudget;  // pairs of pass 1 per tile in plain frames
 constexpr uint32_t kChunk = kBlendChunk;    // pairs per pass-2 chunk
 constexpr size_t kChunkGrid = 8192;         // CTAs of the chunk and fix-up grids at most
-static_assert(kBwdChunk % kBlendThreads == 0, "backward chunk boundaries fall on batch starts");
+constexpr int kBlocks = kTile * kTile / 32;  // 8x4 blocks per tile
+constexpr int kWalkCtas = 5;                // resident CTAs per SM of the walking kernels (48 registers)
+constexpr float kAlphaMin = 1.0f / 255.0f;
+constexpr float kClosed = 2.0f;             // alpha threshold of a pixel that takes no more splats
+constexpr float kStopped = 3.0f;            // the same, stopped inside the current group of pairs
+static_assert(kBwdChunk == kChunk && kTrainBudget % kBwdChunk == 0, "backward chunk boundaries fall on group starts");
 
 // e^q evaluated as 2^(q log2 e) on the hardware ex2 unit
 __device__ __forceinline__ float ex2_approx(float x) {
@@ -59,180 +62,377 @@ __device__ __forceinline__ float ex2_approx(float x) {
     return y;
 }
 
-struct StagedRecord {
-    float4 q, a, c;  // {reach x, reach y, log2 o, C}, {u, v, A, B}, {r, g, b, radius}
-    uint32_t s;         // splat id
-    bool have;
-};
-
-__device__ __forceinline__ void load_record(StagedRecord &r, const uint32_t *__restrict__ pval,
-                                            const float4 *__restrict__ rec, uint32_t idx, uint32_t end) {
-    r.have = idx < end;
-    if (r.have) {
-        r.s = __ldg(pval + idx);
-        const float4 *p = rec + (size_t)r.s * kRecVec;
-        r.q = __ldg(p + 0);
-        r.a = __ldg(p + 1);
-        r.c = __ldg(p + 2);
-    }
+// Two FP32 values in one 64-bit register: the packed instructions round each
+// half exactly as the scalar ones do, at half the issue slots.
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 pack2(float lo, float hi) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float lo2(f2 v) { return __uint_as_float((uint32_t)v); }
+__device__ __forceinline__ float hi2(f2 v) { return __uint_as_float((uint32_t)(v >> 32)); }
+__device__ __forceinline__ f2 add2(f2 a, f2 b) {
+    f2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
+    f2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+    f2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
 }
 
-// kT threads stage batches of kT splats, double-buffered
-template <int kT = kBlendThreads>
-struct BlendShared {
-    // staged splats: {u, v, a', b'}, {c', log2 o, radius, -}, {r, g, b, -} with
-    // p = q log2 e = a' dx^2 + b' dx dy + c' dy^2
-    float4 s0[2][kT];
-    float4 s1[2][kT];
-    float4 s2[2][kT];
-    uint32_t sid[2][kT];
-    uint8_t mask[2][kT];
+// The splats of 32 consecutive pairs that meet a block, compacted in depth
+// order, two neighbours side by side so that one 16-byte load feeds two
+// packed operands.  p = q log2 e = a' dx^2 + b' dx dy + c' dy^2.
+struct __align__(16) HitStage {
+    ulonglong2 uv[16];  // -u, -v
+    ulonglong2 ab[16];  // a', b'
+    ulonglong2 cl[16];  // c', log2 o
+    ulonglong2 rr[16];  // radius, r
+    ulonglong2 gb[16];  // g, b
+    uint32_t id[32];    // splat id (statistics) or one past the pair's index (training)
 };
+
+__device__ __forceinline__ void put2(ulonglong2 *dst, int pos, float first, float second) {
+    float *f = reinterpret_cast<float *>(dst) + (pos >> 1) * 4 + (pos & 1);
+    f[0] = first;
+    f[2] = second;
+}
+
+__device__ __forceinline__ void stage_hit(HitStage &st, int pos, const float4 &q, const float4 &a, const float4 &c) {
+    put2(st.uv, pos, -a.x, -a.y);
+    put2(st.ab, pos, -0.5f * kLog2e * a.z, -kLog2e * a.w);
+    put2(st.cl, pos, -0.5f * kLog2e * q.w, q.z);
+    put2(st.rr, pos, c.w, c.x);
+    put2(st.gb, pos, c.y, c.z);
+}
+
+// A splat that contributes nowhere: fills the last pair of an odd count.
+__device__ __forceinline__ void stage_pad(HitStage &st, int pos) {
+    put2(st.uv, pos, 0.0f, 0.0f);
+    put2(st.ab, pos, 0.0f, 0.0f);
+    put2(st.cl, pos, 0.0f, 0.0f);
+    put2(st.rr, pos, -1.0f, 0.0f);
+    put2(st.gb, pos, 0.0f, 0.0f);
+    st.id[pos] = 0u;
+}
 
 struct Pixel {
-    float T, r, g, b;
-    uint32_t last;  // one past the last composited pair (training forward)
-    bool done;     // saturated, outside the image, or not composited here
-    bool stopped;  // met the stop rule in this call
+    f2 x, y;         // pixel centre, in both halves
+    float T, thr;    // transmittance; smallest alpha that counts (above 1: the pixel takes no more splats)
+    float T0, P;     // T before the current group of pairs; product of 1 - alpha over the group so far
+    f2 r, g, b;      // colour sums of the even and the odd hits
+    uint32_t last;   // one past the last composited pair (training)
 };
 
-// Composite pairs [start, end) of a tile into the calling thread's pixel.
-// Every thread of the CTA must call it with the same range.  kMode 1
-// (statistics): also add each composited weight alpha * T to
-// contrib[splat]; kMode 2 (training): also track the last composited pair.
-// kT: threads of the CTA, covering kT / 32 of the tile's 8x4 warp blocks
-// from block row brow0 (a 16x16 tile has 8: two columns, four rows).
-template <int kMode = 0, int kT = kBlendThreads>
-__device__ __forceinline__ void composite_range(BlendShared<kT> &sh, uint32_t start, uint32_t end,
-                                                const uint32_t *__restrict__ pval,
-                                                const float4 *__restrict__ rec, int tx0, int ty0,
-                                                float fpx, float fpy, Pixel &px,
-                                                float *__restrict__ contrib = nullptr, int brow0 = 0) {
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const uint32_t wbit = 1u << warp;
-    auto stage = [&](const StagedRecord &r, int h) {
-        uint32_t m = 0;
-        if (r.have) {
-            const uint32_t rx = __float_as_uint(r.q.x), ry = __float_as_uint(r.q.y);
-            const int x0 = (int)(rx & 0xFFFFu) - tx0, x1 = (int)(rx >> 16) - tx0;
-            const int y0 = (int)(ry & 0xFFFFu) - ty0, y1 = (int)(ry >> 16) - ty0;
+__device__ __forceinline__ Pixel make_pixel(float x, float y, bool open, const float4 &s, uint32_t last) {
+    return Pixel{pack2(x, x), pack2(y, y), s.w, open ? kAlphaMin : kClosed, s.w, 1.0f, pack2(s.x, 0.0f),
+                 pack2(s.y, 0.0f), pack2(s.z, 0.0f), last};
+}
+__device__ __forceinline__ bool closed(const Pixel &p) { return p.thr > 1.0f; }
+// r, g, b and w
+__device__ __forceinline__ float4 pixel_state(const Pixel &p, float w) {
+    return make_float4(lo2(p.r) + hi2(p.r), lo2(p.g) + hi2(p.g), lo2(p.b) + hi2(p.b), w);
+}
+
+__device__ __forceinline__ float keep_alpha(float dx, float dy, float radius, float p, float e, float thr) {
+    const float alpha = fminf(0.99f, ex2_approx(e));
+    return fmaxf(fabsf(dx), fabsf(dy)) > radius || p > 0.0f || alpha < thr ? 0.0f : alpha;
+}
+
+// alpha of hits 2k and 2k + 1 at the pixel, 0 where a splat does not
+// contribute (outside its support box, q > 0, alpha below the threshold):
+// compositing alpha = 0 leaves T and C unchanged exactly, so no test follows.
+__device__ __forceinline__ void pair_alpha(const HitStage &st, int k, const Pixel &px, float &a0, float &a1) {
+    const ulonglong2 uv = st.uv[k], ab = st.ab[k], cl = st.cl[k];
+    const f2 rad = st.rr[k].x;
+    const f2 dx = add2(px.x, uv.x), dy = add2(px.y, uv.y);
+    const f2 p = fma2(mul2(cl.x, dy), dy, mul2(dx, fma2(ab.y, dy, mul2(ab.x, dx))));
+    const f2 e = add2(p, cl.y);
+    a0 = keep_alpha(lo2(dx), lo2(dy), lo2(rad), lo2(p), lo2(e), px.thr);
+    a1 = keep_alpha(hi2(dx), hi2(dy), hi2(rad), hi2(p), hi2(e), px.thr);
+}
+
+// The same for one splat.
+__device__ __forceinline__ float splat_alpha(float dx, float dy, float a, float b, float c, float lo, float radius) {
+    const float p = __fmaf_rn(__fmul_rn(c, dy), dy, __fmul_rn(dx, __fmaf_rn(b, dy, __fmul_rn(a, dx))));
+    return keep_alpha(dx, dy, radius, p, __fadd_rn(p, lo), kAlphaMin);
+}
+
+__device__ __forceinline__ void add_colour(const HitStage &st, int k, Pixel &px, f2 w) {
+    const ulonglong2 gb = st.gb[k];
+    px.r = fma2(st.rr[k].y, w, px.r);
+    px.g = fma2(gb.x, w, px.g);
+    px.b = fma2(gb.y, w, px.b);
+}
+
+// kMode 0: colour only; 1 (statistics): also add every composited weight
+// alpha T, summed over the warp's pixels, to contrib[splat]; 2 (training):
+// also track the last composited pair.
+enum { kPlain = 0, kStats = 1, kTraining = 2 };
+
+// The staged hits composited in order, with the stop rule.  Every lane of
+// the warp calls it.
+template <int kMode>
+__device__ __forceinline__ void walk_hits(const HitStage &st, int cnt, Pixel &px, float *__restrict__ contrib) {
+#pragma unroll 1
+    for (int k = 0; 2 * k < cnt; ++k) {
+        float a0, a1;
+        pair_alpha(st, k, px, a0, a1);
+        const float o0 = 1.0f - a0, o1 = 1.0f - a1, P1 = px.P * o0;
+        float T1 = px.T * o0, T2 = T1 * o1;
+        if (kMode == kTraining) px.P = P1 * o1;
+        if (__any_sync(0xffffffffu, T2 < 1e-4f)) {
+            // some pixel stops at one of the two (closed ones keep their T)
+            if (T1 < 1e-4f) {
+                a0 = a1 = 0.0f;
+                T1 = T2 = px.T;
+                if (kMode == kTraining) px.P = P1;
+                px.thr = kStopped;
+            } else if (T2 < 1e-4f) {
+                a1 = 0.0f;
+                T2 = T1;
+                px.thr = kStopped;
+            }
+        }
+        const float w0 = a0 * px.T, w1 = a1 * T1;
+        add_colour(st, k, px, pack2(w0, w1));
+        px.T = T2;
+        if (kMode == kTraining) {
+            if (a0 > 0.0f) px.last = st.id[2 * k];
+            if (a1 > 0.0f) px.last = st.id[2 * k + 1];
+        }
+        if (kMode == kStats && __any_sync(0xffffffffu, w0 + w1 > 0.0f)) {
+            // both sums in five exchanges: each half warp takes one splat
+            const bool up = (threadIdx.x & 16) != 0;
+            float v = (up ? w1 : w0) + __shfl_xor_sync(0xffffffffu, up ? w0 : w1, 16);
 #pragma unroll
-            for (int w = 0; w < kT / 32; ++w) {
-                const int bx = (w & 1) * kBlockW, by = ((w >> 1) + brow0) * kBlockH;
-                if (x0 <= bx + kBlockW - 1 && x1 >= bx && y0 <= by + kBlockH - 1 && y1 >= by) m |= 1u << w;
-            }
-            sh.s0[h][tid] = make_float4(r.a.x, r.a.y, -0.5f * kLog2e * r.a.z, -kLog2e * r.a.w);
-            sh.s1[h][tid] = make_float4(-0.5f * kLog2e * r.q.w, r.q.z, r.c.w, 0.0f);
-            sh.s2[h][tid] = r.c;
-            if (kMode == 1) sh.sid[h][tid] = r.s;
+            for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if ((threadIdx.x & 15) == 0 && v > 0.0f) atomicAdd(contrib + st.id[2 * k + (up ? 1 : 0)], v);
         }
-        sh.mask[h][tid] = (uint8_t)m;
-    };
-    // the buffers may still be read by a previous call; leave when no pixel is open
-    if (__syncthreads_count(px.done) == kT || start >= end) return;
-    StagedRecord nxt;
-    load_record(nxt, pval, rec, start + tid, end);
-    stage(nxt, 0);
-    load_record(nxt, pval, rec, start + kT + tid, end);
-    __syncthreads();
-    int h = 0;
-    for (uint32_t base = start; base < end; base += kT, h ^= 1) {
-        const int nb = (int)min((uint32_t)kT, end - base);
-        for (int c = 0; c < nb; c += 32) {
-            if (__all_sync(0xffffffffu, px.done)) break;
-            const bool mine = (sh.mask[h][c + lane] & wbit) != 0 && c + lane < nb;
-            uint32_t m = __ballot_sync(0xffffffffu, mine);
-            while (m) {
-                const int j = c + __ffs(m) - 1;
-                m &= m - 1;
-                if (px.done) continue;
-                const float4 a = sh.s0[h][j];  // u, v, a', b'
-                const float4 b = sh.s1[h][j];  // c', log2 o, radius
-                const float dx = fpx - a.x, dy = fpy - a.y;
-                if (fmaxf(fabsf(dx), fabsf(dy)) > b.z) continue;
-                const float p = dx * (a.z * dx + a.w * dy) + b.x * dy * dy;
-                if (p > 0.0f) continue;
-                const float alpha = fminf(0.99f, ex2_approx(p + b.y));
-                if (alpha < (1.0f / 255.0f)) continue;
-                const float Tn = px.T * (1.0f - alpha);
-                if (Tn < 1e-4f) {
-                    px.done = true;
-                    px.stopped = true;
-                    continue;
-                }
-                const float4 col = sh.s2[h][j];
-                const float wgt = alpha * px.T;
-                if (kMode == 1) atomicAdd(contrib + sh.sid[h][j], wgt);
-                if (kMode == 2) px.last = base + (uint32_t)j + 1u;
-                px.r += col.x * wgt;
-                px.g += col.y * wgt;
-                px.b += col.z * wgt;
-                px.T = Tn;
-            }
-        }
-        // the other half was last read before the previous barrier: refill it
-        // with the next batch (loaded while this one was composited) and
-        // start loading the batch after
-        if (base + kT < end) {
-            stage(nxt, h ^ 1);
-            load_record(nxt, pval, rec, base + 2 * kT + tid, end);
-        }
-        if (__syncthreads_count(px.done) == kT) break;
     }
 }
 
-struct TileGeom {
-    int tx0, ty0, px, py;
+// Lane's pair as loaded ahead: its splat and first record word.
+__device__ __forceinline__ bool meets_block(const float4 &q, int bx0, int by0) {
+    const uint32_t rx = __float_as_uint(q.x), ry = __float_as_uint(q.y);
+    return (int)(rx & 0xFFFFu) <= bx0 + kBlockW - 1 && (int)(rx >> 16) >= bx0 &&
+           (int)(ry & 0xFFFFu) <= by0 + kBlockH - 1 && (int)(ry >> 16) >= by0;
+}
+
+// Stage the lanes' pairs whose reach box meets the block; returns how many.
+// Only those load the other 32 bytes of their record.
+template <int kMode>
+__device__ __forceinline__ int stage_hits(HitStage &st, bool have, uint32_t s, const float4 &q, uint32_t pair,
+                                          const float4 *__restrict__ rec, int bx0, int by0) {
+    const int lane = threadIdx.x & 31;
+    const bool mine = have && meets_block(q, bx0, by0);
+    const uint32_t m = __ballot_sync(0xffffffffu, mine);
+    const int cnt = __popc(m);
+    if (mine) {
+        const float4 *p = rec + (size_t)s * kRecVec;
+        const float4 a = __ldg(p + 1), c = __ldg(p + 2);
+        const int pos = __popc(m & ((1u << lane) - 1u));
+        stage_hit(st, pos, q, a, c);
+        if (kMode != kPlain) st.id[pos] = kMode == kStats ? s : pair + 1u;
+    }
+    if (lane == 0 && (cnt & 1)) stage_pad(st, cnt);
+    return cnt;
+}
+
+// Training: what a pixel keeps for the backward, its final state and one
+// past its last composited pair.
+__device__ __forceinline__ void store_final(const BlendWork &work, size_t pix, uint32_t last, const float4 &s) {
+    work.px_end[pix] = last;
+    work.px_fin[pix] = s;
+}
+
+// Training: an open pixel's state before pair `base` of the tile's list, at
+// every kBwdChunk-th pair (p: the pixel's number in its tile).
+__device__ __forceinline__ void store_boundary(const BlendWork &work, uint32_t start, uint32_t base, int p,
+                                               const float4 &s) {
+    if (base > start && (base - start) % kBwdChunk == 0)
+        work.px_bnd[(size_t)(base / kBwdChunk) * kBlendThreads + p] = s;
+}
+
+// The pixel stopped inside the group by its pair-by-pair T, but not by T0 P
+// (one rounding apart).  The group's whole product decides: below the
+// threshold, the pixel stays stopped where it is; otherwise it takes the
+// pairs from the stopping one to the group's end as well.  Lanes that come
+// here (one pixel in millions) read the group's pairs [g0, g1) again.
+__device__ __noinline__ void settle_stop(Pixel &px, uint32_t g0, uint32_t g1, const uint32_t *__restrict__ pval,
+                                         const float4 *__restrict__ rec) {
+    float P = 1.0f, T = px.T0, Ts = 0.0f, r = 0.0f, g = 0.0f, b = 0.0f;
+    uint32_t last = px.last;
+    bool past = false;
+    for (uint32_t i = g0; i < g1; ++i) {
+        const uint32_t s = __ldg(pval + i);
+        const float4 *p = rec + (size_t)s * kRecVec;
+        const float4 q = __ldg(p), a = __ldg(p + 1), c = __ldg(p + 2);
+        const float alpha = splat_alpha(lo2(px.x) - a.x, lo2(px.y) - a.y, -0.5f * kLog2e * a.z, -kLog2e * a.w,
+                                        -0.5f * kLog2e * q.w, q.z, c.w);
+        P *= 1.0f - alpha;
+        const float Tn = T * (1.0f - alpha);
+        if (!past && Tn < 1e-4f) {
+            past = true;
+            Ts = T;
+        }
+        if (past && alpha > 0.0f) {
+            const float w = alpha * T;
+            r += c.x * w;
+            g += c.y * w;
+            b += c.z * w;
+            last = i + 1u;
+        }
+        T = Tn;
+    }
+    const float Tq = px.T0 * P;
+    if (Tq < 1e-4f) {
+        px.T = Ts;
+        px.thr = kClosed;
+        return;
+    }
+    px.T = Tq;
+    px.thr = kAlphaMin;
+    px.last = last;
+    px.r = add2(px.r, pack2(r, 0.0f));
+    px.g = add2(px.g, pack2(g, 0.0f));
+    px.b = add2(px.b, pack2(b, 0.0f));
+}
+
+// End of the group of pairs [g0, g1): T is T0 times the group's product
+// where that stays above the stop threshold, the pair-by-pair T (and where it
+// stopped) otherwise.
+__device__ __forceinline__ void settle_group(Pixel &px, uint32_t g0, uint32_t g1, const uint32_t *__restrict__ pval,
+                                             const float4 *__restrict__ rec) {
+    const float Tq = px.T0 * px.P;
+    const bool stopped = px.thr == kStopped;
+    if (Tq >= 1e-4f) {
+        if (stopped) {
+            Pixel t = px;  // a copy: the pixel itself stays in registers
+            settle_stop(t, g0, g1, pval, rec);
+            px = t;
+        } else if (!closed(px)) {
+            px.T = Tq;
+        }
+    } else if (stopped) {
+        px.thr = kClosed;
+    }
+    px.T0 = px.T;
+    px.P = 1.0f;
+}
+
+// The warp's block composited over pairs [start, end), 32 at a time; the
+// splat ids are loaded two batches ahead and the reach boxes one, so that
+// only the hits' records are waited for.  With `groups` (training),
+// T is settled every kChunk pairs from start and each open pixel's state
+// kept where they begin; without, T is the pair-by-pair product.
+template <int kMode>
+__device__ __forceinline__ void warp_walk(HitStage &st, uint32_t start, uint32_t end, const uint32_t *__restrict__ pval,
+                                          const float4 *__restrict__ rec, int bx0, int by0, Pixel &px,
+                                          const BlendWork &work, bool groups) {
+    const int lane = threadIdx.x & 31;
+    if (start >= end || __all_sync(0xffffffffu, closed(px))) return;
+    uint32_t i = start + (uint32_t)lane;
+    uint32_t s = i < end ? __ldg(pval + i) : 0u;
+    uint32_t s1 = i + 32u < end ? __ldg(pval + i + 32) : 0u;
+    float4 q = i < end ? __ldg(rec + (size_t)s * kRecVec) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+    for (uint32_t base = start; base < end; base += 32u, i += 32u) {
+        if (kMode == kTraining && groups && !closed(px))
+            store_boundary(work, start, base, (int)threadIdx.x, pixel_state(px, px.T));
+        const int cnt = stage_hits<kMode>(st, i < end, s, q, i, rec, bx0, by0);
+        s = s1;
+        if (i + 32u < end) q = __ldg(rec + (size_t)s * kRecVec);
+        if (i + 64u < end) s1 = __ldg(pval + i + 64);
+        __syncwarp();
+        walk_hits<kMode>(st, cnt, px, work.contrib);
+        __syncwarp();  // the staging buffer is refilled by the next batch
+        const uint32_t next = base + 32u;
+        bool settled = true;
+        if (kMode == kTraining && groups) {
+            if (next >= end || (next - start) % kChunk == 0u)
+                settle_group(px, next - 1u - (next - 1u - start) % kChunk, min(next, end), pval, rec);
+            settled = px.thr != kStopped || px.T0 * px.P < 1e-4f;
+        }
+        if (__all_sync(0xffffffffu, closed(px) && settled)) break;
+    }
+}
+
+struct BlockGeom {
+    int bx0, by0, px, py;
     bool inside;
     float fpx, fpy;
 };
 
-// Pixel of the calling thread: warp w of the tile (w0 = the CTA's first)
-// covers the 8x4 block at column w % 2, row w / 2.
-__device__ __forceinline__ TileGeom tile_geom(int tile, int tiles_x, int W, int H, int ox, int oy, int w0 = 0) {
-    TileGeom g;
-    const int tyi = tile / tiles_x, txi = tile - tyi * tiles_x;
-    const int warp = w0 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    g.tx0 = txi * kTile;
-    g.ty0 = tyi * kTile;
-    g.px = g.tx0 + (warp & 1) * kBlockW + (lane & (kBlockW - 1));
-    g.py = g.ty0 + (warp >> 1) * kBlockH + (lane / kBlockW);
+// Block blk of a tile (column blk % 2, row blk / 2) and the lane's pixel.
+__device__ __forceinline__ BlockGeom block_geom(int tile, int blk, int tiles_x, int W, int H, int ox, int oy) {
+    BlockGeom g;
+    const int tyi = tile / tiles_x, txi = tile - tyi * tiles_x, lane = threadIdx.x & 31;
+    g.bx0 = txi * kTile + (blk & 1) * kBlockW;
+    g.by0 = tyi * kTile + (blk >> 1) * kBlockH;
+    g.px = g.bx0 + (lane & (kBlockW - 1));
+    g.py = g.by0 + lane / kBlockW;
     g.inside = g.px < W && g.py < H;
     g.fpx = (float)(g.px + ox) + 0.5f;
     g.fpy = (float)(g.py + oy) + 0.5f;
     return g;
 }
 
-// One CTA per tile: the first kBudget pairs of the tile (kMode 1,
-// statistics: every pair in one pass).  kT threads per CTA: 256 cover a tile,
-// 128 half a tile (two CTAs per tile, rows 0-7 and 8-15, each compositing
-// the tile's list on its own, so the halves do not wait for each other).
-template <int kMode, int kT>
-__global__ void __launch_bounds__(kT) k_blend(int tiles_x, int W, int H, const uint2 *__restrict__ ranges,
-                                              const uint32_t *__restrict__ pval, const float4 *__restrict__ rec,
-                                              float4 *__restrict__ out, BlendWork work) {
-    __shared__ BlendShared<kT> sh;
-    constexpr int kParts = kBlendThreads / kT;
-    const int tile = blockIdx.x / kParts, part = blockIdx.x % kParts;
-    const int w0 = part * (kT / 32);  // first warp block of this CTA
-    const TileGeom g = tile_geom(tile, tiles_x, W, H, work.ox, work.oy, w0);
+// The pixel's state at the start of the split passes (T negated when closed).
+__device__ __forceinline__ void keep_state(const BlendWork &work, int slot, const Pixel &px, bool open) {
+    const size_t sp = (size_t)slot * kBlendThreads + threadIdx.x;
+    work.state[sp] = pixel_state(px, open ? px.T : -px.T);
+    work.slast[sp] = px.last;
+    if (open) work.cand_done[slot] = 0u;  // any of them: the plan set it to 1
+}
+
+// Statistics frames (every list to its end) and the first kTrainBudget pairs
+// of training frames: a CTA per tile, tiles in decreasing list length class,
+// a warp per block.  The warps share nothing but the cache lines of the
+// tile's records: no CTA barrier, so a warp whose block saturates early waits
+// for nobody, and only pairs in front of the saturating one are evaluated.
+// Bound by instruction issue (68% of the slots at 52% of the warps).  Against
+// a CTA of eight warps in step over batches of 256 pairs (stalled 13 of 22
+// cycles at its barriers, one atomic per pixel and splat): statistics frame
+// of 100 full-detail characters at 3840x2160 2.63 -> 2.05 ms (this kernel
+// 1.91 -> 1.18).  Against chunks of kChunk pairs composited in parallel from
+// T = 1, which evaluates the hidden ones too: training frame of 64
+// characters at 512x512 1.52 -> 0.69 ms of compositing.  48 registers and 40
+// warps per SM are faster than 40 and 48 (spills) or 32 and 64.
+template <int kMode>
+__global__ void __launch_bounds__(kBlendThreads, kWalkCtas) k_blend_walk(int tiles_x, int W, int H,
+                                                                         const uint2 *__restrict__ ranges,
+                                                                         const uint32_t *__restrict__ pval,
+                                                                         const float4 *__restrict__ rec,
+                                                                         float4 *__restrict__ out, BlendWork work) {
+    __shared__ HitStage st[kBlocks];
+    const int tile = work.pp_tile[blockIdx.x], warp = threadIdx.x >> 5;
+    if (!in_bounds(tile < tiles_x * ((H + kTile - 1) / kTile), kChkTile)) return;
+    const BlockGeom g = block_geom(tile, warp, tiles_x, W, H, work.ox, work.oy);
+    const size_t pix = (size_t)g.py * W + g.px;
     uint2 rg = ranges[tile];
     if (!in_bounds(rg.x <= rg.y && rg.y <= work.n_pairs, kChkPair)) rg.y = rg.x;
-    Pixel px{1.0f, 0.0f, 0.0f, 0.0f, rg.x, !g.inside, false};
-    const uint32_t end1 = rg.y - rg.x > kBudget && kMode == 0 ? rg.x + kBudget : rg.y;
-    composite_range<kMode, kT>(sh, rg.x, end1, pval, rec, g.tx0, g.ty0, g.fpx, g.fpy, px, work.contrib, w0 / 2);
-    if (end1 < rg.y && in_bounds(work.cand_slot[tile] >= 0, kChkSlot)) {
-        // pairs remain: record the pixel state for pass 2 and the merge (the
-        // plan set cand_done to 1; every part clears it unless all its
-        // pixels are done)
-        const int slot = work.cand_slot[tile];
-        const int all = __syncthreads_count(px.done) == kT;
-        if (threadIdx.x == 0 && !all) atomicAnd(work.cand_done + slot, 0u);
-        work.state[(size_t)slot * kBlendThreads + part * kT + threadIdx.x] =
-            make_float4(px.r, px.g, px.b, px.done ? -px.T : px.T);
-        if (!all) return;
+    const uint32_t n = rg.y - rg.x, end = rg.x + (kMode == kStats ? n : min(n, work.budget));
+    Pixel px = make_pixel(g.fpx, g.fpy, g.inside, make_float4(0.f, 0.f, 0.f, 1.f), n ? rg.x : 0u);
+    warp_walk<kMode>(st[warp], rg.x, end, pval, rec, g.bx0, g.by0, px, work, kMode == kTraining);
+    if (kMode == kTraining && end < rg.y && in_bounds(work.cand_slot[tile] >= 0, kChkSlot)) {
+        // the merge reads the whole tile's states
+        const bool open = !closed(px), any = __any_sync(0xffffffffu, open);
+        keep_state(work, work.cand_slot[tile], px, open);
+        if (any) return;
     }
-    if (g.inside) out[(size_t)g.py * W + g.px] = make_float4(px.r, px.g, px.b, 1.0f - px.T);
+    if (g.inside) {
+        out[pix] = pixel_state(px, 1.0f - px.T);
+        if (kMode == kTraining) store_final(work, pix, px.last, pixel_state(px, px.T));
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -270,7 +470,7 @@ constexpr int kPpTileClass = 14;               // lists of fewer than 8,192 pair
 static_assert((1u << (kPpTileClass - 1)) <= kBlendBudget, "a tile item composites its whole list");
 
 struct PpShared {
-    float4 s0[kPpWarps][32];  // u, v, a', b' (as staged by composite_range)
+    float4 s0[kPpWarps][32];  // u, v, a', b' with p = q log2 e = a' dx^2 + b' dx dy + c' dy^2
     float4 s1[kPpWarps][32];  // c', log2 o, radius, -
     float4 s2[kPpWarps][32];  // r, g, b, -
     float4 part[kPpWarps][32];
@@ -349,8 +549,7 @@ __device__ __forceinline__ bool key_segments(const int32_t *__restrict__ meta, i
 }
 
 // alpha of a staged splat at a pixel centre; 0 when the splat does not
-// contribute there (outside its support box, q > 0, alpha < 1/255).  The
-// same arithmetic as composite_range.  kBranchFree evaluates every test
+// contribute there (outside its support box, q > 0, alpha < 1/255).  kBranchFree evaluates every test
 // without branches: a splat that does not contribute then leaves T and C
 // unchanged when composited with alpha = 0 (T (1 - 0) = T exactly), so the
 // caller needs no test either.  That pays where the pairs of a sub-range
@@ -608,53 +807,57 @@ __global__ void __launch_bounds__(kPpThreads, 8) k_blend_pp(int tiles_x, int W, 
     }
 }
 
-// Pass 2: chunk c of a tile's remaining pairs, from T = 1, for the pixels
-// pass 1 left open.  Writes (r, g, b, T) with T negated when the chunk met
-// the stop rule.
-__global__ void __launch_bounds__(kBlendThreads) k_blend_chunks(int tiles_x, int W, int H,
-                                                                const uint2 *__restrict__ ranges,
-                                                                const uint32_t *__restrict__ pval,
-                                                                const float4 *__restrict__ rec,
-                                                                BlendWork work) {
-    __shared__ BlendShared<> sh;
+// Chunk c of a tile's pairs past the budget, from T = 1, for the pixels still
+// open; a warp per block.  Writes (r, g, b, T) with T negated when the chunk
+// met the stop rule.
+template <bool kTrain>
+__global__ void __launch_bounds__(kBlendThreads, kWalkCtas) k_blend_chunks(int tiles_x, int W, int H,
+                                                                           const uint2 *__restrict__ ranges,
+                                                                           const uint32_t *__restrict__ pval,
+                                                                           const float4 *__restrict__ rec,
+                                                                           BlendWork work) {
+    __shared__ HitStage st[kBlocks];
+    const int warp = threadIdx.x >> 5;
     // chunk w of the frame, grid-stride (the grid is capped, not sized for
     // the worst case)
     for (uint32_t w = blockIdx.x; w < (uint32_t)work.meta[1]; w += gridDim.x) {
         const int slot = work.chunk_slot[w];
         if (work.cand_done[slot]) continue;
         const int tile = work.cand_tile[slot];
-        const TileGeom g = tile_geom(tile, tiles_x, W, H, work.ox, work.oy);
+        const BlockGeom g = block_geom(tile, warp, tiles_x, W, H, work.ox, work.oy);
         const uint2 rg = ranges[tile];
         if (!in_bounds(rg.y <= work.n_pairs, kChkPair)) continue;
-        const uint32_t c = w - work.cand_chunk0[slot];
-        const uint32_t start = rg.x + kBudget + c * kChunk;
-        const uint32_t end = min(rg.y, start + kChunk);
-        const float4 s1 = work.state[(size_t)slot * kBlendThreads + threadIdx.x];
-        Pixel px{1.0f, 0.0f, 0.0f, 0.0f, 0u, !g.inside || s1.w < 0.0f, false};
-        composite_range(sh, start, end, pval, rec, g.tx0, g.ty0, g.fpx, g.fpy, px);
-        work.part[(size_t)w * kBlendThreads + threadIdx.x] = make_float4(px.r, px.g, px.b, px.stopped ? -px.T : px.T);
-        __syncthreads();  // the staging buffers are reused by the next chunk
+        const uint32_t start = rg.x + work.budget + (w - work.cand_chunk0[slot]) * kChunk;
+        const bool open = g.inside && work.state[(size_t)slot * kBlendThreads + threadIdx.x].w >= 0.0f;
+        Pixel px = make_pixel(g.fpx, g.fpy, open, make_float4(0.f, 0.f, 0.f, 1.f), 0u);
+        warp_walk<kTrain ? kTraining : kPlain>(st[warp], start, min(rg.y, start + kChunk), pval, rec, g.bx0, g.by0, px,
+                                               work, false);
+        work.part[(size_t)w * kBlendThreads + threadIdx.x] = pixel_state(px, open && closed(px) ? -px.T : px.T);
+        if (kTrain) work.last[(size_t)w * kBlendThreads + threadIdx.x] = px.last;
+        __syncwarp();  // the staging buffer is reused by the next chunk
     }
 }
 
-// Merge: pass-1 state then the chunks in depth order, per pixel, up to the
+// Merge: the state at the budget, then the chunks in depth order, per pixel, up to the
 // chunk in which the pixel meets the stop rule: such pixels keep their
 // state before that chunk (in work.state) and its index (work.stop) for the
 // fix-up pass; the others are final.
+template <bool kTrain>
 __global__ void __launch_bounds__(kBlendThreads) k_blend_merge(int tiles_x, int W, int H,
                                                                const uint2 *__restrict__ ranges,
                                                                float4 *__restrict__ out, BlendWork work) {
     const int slot = blockIdx.x;
     if (slot >= work.meta[0] || work.cand_done[slot]) return;
     const int tile = work.cand_tile[slot];
-    const TileGeom g = tile_geom(tile, tiles_x, W, H, work.ox, work.oy);
+    const BlockGeom g = block_geom(tile, threadIdx.x >> 5, tiles_x, W, H, work.ox, work.oy);
     const size_t pix = (size_t)slot * kBlendThreads + threadIdx.x;
     const float4 s1 = work.state[pix];
     float T = fabsf(s1.w), r = s1.x, gg = s1.y, b = s1.z;
     bool done = !g.inside || s1.w < 0.0f;
+    uint32_t last = kTrain ? work.slast[pix] : 0u;
     int32_t stop = -1;
     const uint2 rg = ranges[tile];
-    const uint32_t c0 = work.cand_chunk0[slot], c1 = c0 + (rg.y - rg.x - kBudget + kChunk - 1) / kChunk;
+    const uint32_t c0 = work.cand_chunk0[slot], c1 = c0 + (rg.y - rg.x - work.budget + kChunk - 1) / kChunk;
     // four chunks' partials loaded at a time (independent loads), applied in order
     for (uint32_t w0 = c0; w0 < c1 && !done; w0 += 4) {
         float4 pk[4];
@@ -664,6 +867,7 @@ __global__ void __launch_bounds__(kBlendThreads) k_blend_merge(int tiles_x, int 
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             if (done || w0 + i >= c1) break;
+            if (kTrain) store_boundary(work, rg.x, rg.x + work.budget + (w0 + i - c0) * kChunk, (int)threadIdx.x, make_float4(r, gg, b, T));
             const float Tk = fabsf(pk[i].w);
             if (T * Tk >= 1e-4f) {
                 // no splat of the chunk reaches the stop rule from this T: the
@@ -672,6 +876,10 @@ __global__ void __launch_bounds__(kBlendThreads) k_blend_merge(int tiles_x, int 
                 gg += T * pk[i].y;
                 b += T * pk[i].z;
                 T *= Tk;
+                if (kTrain) {
+                    const uint32_t lk = work.last[(size_t)(w0 + i) * kBlendThreads + threadIdx.x];
+                    if (lk) last = lk;
+                }
                 done = pk[i].w < 0.0f;
             } else {
                 stop = (int32_t)(w0 + i);
@@ -680,167 +888,53 @@ __global__ void __launch_bounds__(kBlendThreads) k_blend_merge(int tiles_x, int 
         }
     }
     work.stop[pix] = stop;
-    if (stop >= 0) work.state[pix] = make_float4(r, gg, b, T);
-    else if (g.inside) out[(size_t)g.py * W + g.px] = make_float4(r, gg, b, 1.0f - T);
+    if (stop >= 0) {
+        work.state[pix] = make_float4(r, gg, b, T);
+        if (kTrain) work.slast[pix] = last;
+    } else if (g.inside) {
+        out[(size_t)g.py * W + g.px] = make_float4(r, gg, b, 1.0f - T);
+        if (kTrain) store_final(work, (size_t)g.py * W + g.px, last, make_float4(r, gg, b, T));
+    }
 }
 
 // Fix-up: chunk w composited again, from their true transmittance, for the
 // pixels that meet the stop rule inside it.
-__global__ void __launch_bounds__(kBlendThreads) k_blend_fix(int tiles_x, int W, int H,
-                                                             const uint2 *__restrict__ ranges,
-                                                             const uint32_t *__restrict__ pval,
-                                                             const float4 *__restrict__ rec,
-                                                             float4 *__restrict__ out, BlendWork work) {
-    __shared__ BlendShared<> sh;
+template <bool kTrain>
+__global__ void __launch_bounds__(kBlendThreads, kWalkCtas) k_blend_fix(int tiles_x, int W, int H,
+                                                                        const uint2 *__restrict__ ranges,
+                                                                        const uint32_t *__restrict__ pval,
+                                                                        const float4 *__restrict__ rec,
+                                                                        float4 *__restrict__ out, BlendWork work) {
+    __shared__ HitStage st[kBlocks];
+    const int warp = threadIdx.x >> 5;
     for (uint32_t w = blockIdx.x; w < (uint32_t)work.meta[1]; w += gridDim.x) {
         const int slot = work.chunk_slot[w];
         if (work.cand_done[slot]) continue;
-        const size_t pix = (size_t)slot * kBlendThreads + threadIdx.x;
-        const bool mine = work.stop[pix] == (int32_t)w;
-        if (__syncthreads_count(mine) == 0) continue;
+        const size_t sp = (size_t)slot * kBlendThreads + threadIdx.x;
+        const bool mine = work.stop[sp] == (int32_t)w;
+        if (!__any_sync(0xffffffffu, mine)) continue;
         const int tile = work.cand_tile[slot];
-        const TileGeom g = tile_geom(tile, tiles_x, W, H, work.ox, work.oy);
+        const BlockGeom g = block_geom(tile, warp, tiles_x, W, H, work.ox, work.oy);
         const uint2 rg = ranges[tile];
         if (!in_bounds(rg.y <= work.n_pairs, kChkPair)) continue;
-        const float4 sb = mine ? work.state[pix] : make_float4(0.f, 0.f, 0.f, 1.f);
-        Pixel px{sb.w, sb.x, sb.y, sb.z, 0u, !mine, false};
-        const uint32_t start = rg.x + kBudget + (w - work.cand_chunk0[slot]) * kChunk;
-        composite_range(sh, start, min(rg.y, start + kChunk), pval, rec, g.tx0, g.ty0, g.fpx, g.fpy, px);
-        if (mine && g.inside) out[(size_t)g.py * W + g.px] = make_float4(px.r, px.g, px.b, 1.0f - px.T);
-        __syncthreads();  // the staging buffers are reused by the next chunk
-    }
-}
-
-// ---------------------------------------------------------------------------
-// Training frames: every tile's list in chunks of kBwdChunk pairs composited
-// in parallel, as the split passes of plain frames do (the operator is
-// associative), and per pixel the state at each chunk boundary, the end of
-// its composited list and its final state for the backward.
-//   k_train_counts   chunks per tile (then an exclusive scan numbers them)
-//   k_train_chunks   CTA per chunk: its composite from T = 1 for every pixel
-//                    of the tile, and one past its last composited pair
-//   k_train_merge    CTA per tile: per pixel, the chunks in order, C += T C_k,
-//                    T *= T_k, keeping the state before every chunk; up to the
-//                    chunk in which T T_k would fall below the stop threshold
-//                    (or whose partial met it from T = 1)
-//   k_train_fix      CTA per chunk: that chunk again from the pixel's true
-//                    state with the stop rule, for the pixels stopping in it
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_train_counts(int n_tiles, const uint2 *__restrict__ ranges,
-                                                      uint32_t *__restrict__ cnt) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < n_tiles) cnt[t] = (ranges[t].y - ranges[t].x + kBwdChunk - 1) / kBwdChunk;
-}
-
-// tile of chunk w: the last t with chunk0[t] <= w (thread 0, broadcast)
-__device__ __forceinline__ int chunk_tile(const uint32_t *__restrict__ chunk0, int n_tiles, uint32_t w, int *s_tile) {
-    if (threadIdx.x == 0) {
-        int lo = 0, hi = n_tiles - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (chunk0[mid] <= w) lo = mid;
-            else hi = mid - 1;
+        Pixel px = make_pixel(g.fpx, g.fpy, mine, mine ? work.state[sp] : make_float4(0.f, 0.f, 0.f, 1.f),
+                              kTrain && mine ? work.slast[sp] : 0u);
+        const uint32_t start = rg.x + work.budget + (w - work.cand_chunk0[slot]) * kChunk;
+        warp_walk<kTrain ? kTraining : kPlain>(st[warp], start, min(rg.y, start + kChunk), pval, rec, g.bx0, g.by0, px,
+                                               work, false);
+        if (mine && g.inside) {
+            const size_t pix = (size_t)g.py * W + g.px;
+            out[pix] = pixel_state(px, 1.0f - px.T);
+            if (kTrain) store_final(work, pix, px.last, pixel_state(px, px.T));
         }
-        *s_tile = lo;
-    }
-    __syncthreads();
-    return *s_tile;
-}
-
-__global__ void __launch_bounds__(kBlendThreads) k_train_chunks(int tiles_x, int W, int H,
-                                                                const uint2 *__restrict__ ranges,
-                                                                const uint32_t *__restrict__ pval,
-                                                                const float4 *__restrict__ rec, BlendWork work) {
-    __shared__ BlendShared<> sh;
-    __shared__ int s_tile;
-    const int n_tiles = tiles_x * ((H + kTile - 1) / kTile);
-    const uint32_t w = blockIdx.x;
-    if (w >= work.t_chunk0[n_tiles]) return;
-    const int tile = chunk_tile(work.t_chunk0, n_tiles, w, &s_tile);
-    const TileGeom g = tile_geom(tile, tiles_x, W, H, work.ox, work.oy);
-    const uint2 rg = ranges[tile];
-    const uint32_t a = rg.x + (w - work.t_chunk0[tile]) * kBwdChunk, b = min(rg.y, a + kBwdChunk);
-    Pixel px{1.0f, 0.0f, 0.0f, 0.0f, 0u, !g.inside, false};
-    composite_range<2>(sh, a, b, pval, rec, g.tx0, g.ty0, g.fpx, g.fpy, px);
-    work.t_part[(size_t)w * kBlendThreads + threadIdx.x] = make_float4(px.r, px.g, px.b, px.stopped ? -px.T : px.T);
-    work.t_last[(size_t)w * kBlendThreads + threadIdx.x] = px.last;
-}
-
-__global__ void __launch_bounds__(kBlendThreads) k_train_merge(int tiles_x, int W, int H,
-                                                               const uint2 *__restrict__ ranges,
-                                                               float4 *__restrict__ out, BlendWork work) {
-    const int tile = blockIdx.x;
-    const TileGeom g = tile_geom(tile, tiles_x, W, H, work.ox, work.oy);
-    if (!g.inside) return;
-    const size_t pix = (size_t)g.py * W + g.px;
-    const uint2 rg = ranges[tile];
-    float T = 1.0f, r = 0.0f, gg = 0.0f, b = 0.0f;
-    uint32_t last = rg.x;
-    int32_t stop = -1;
-    const uint32_t c0 = work.t_chunk0[tile], c1 = work.t_chunk0[tile + 1];
-    for (uint32_t w = c0; w < c1; ++w) {
-        if (w > c0) {
-            // the state before pair a of chunk w, for the backward
-            const uint32_t a = rg.x + (w - c0) * kBwdChunk;
-            work.px_bnd[(size_t)(a / kBwdChunk) * kBlendThreads + threadIdx.x] = make_float4(r, gg, b, T);
-        }
-        const float4 p = work.t_part[(size_t)w * kBlendThreads + threadIdx.x];
-        const float Tk = fabsf(p.w);
-        if (p.w >= 0.0f && T * Tk >= 1e-4f) {
-            // no splat of the chunk meets the stop rule from this T: it applies as a whole
-            r += T * p.x;
-            gg += T * p.y;
-            b += T * p.z;
-            T *= Tk;
-            const uint32_t lk = work.t_last[(size_t)w * kBlendThreads + threadIdx.x];
-            if (lk) last = lk;
-        } else {
-            stop = (int32_t)w;
-            break;
-        }
-    }
-    work.t_stop[pix] = stop;
-    if (stop >= 0) {
-        work.t_state[pix] = make_float4(r, gg, b, T);
-        work.t_slast[pix] = last;
-    } else {
-        out[pix] = make_float4(r, gg, b, 1.0f - T);
-        work.px_end[pix] = last;
-        work.px_fin[pix] = make_float4(r, gg, b, T);
-    }
-}
-
-__global__ void __launch_bounds__(kBlendThreads) k_train_fix(int tiles_x, int W, int H,
-                                                             const uint2 *__restrict__ ranges,
-                                                             const uint32_t *__restrict__ pval,
-                                                             const float4 *__restrict__ rec,
-                                                             float4 *__restrict__ out, BlendWork work) {
-    __shared__ BlendShared<> sh;
-    __shared__ int s_tile;
-    const int n_tiles = tiles_x * ((H + kTile - 1) / kTile);
-    const uint32_t w = blockIdx.x;
-    if (w >= work.t_chunk0[n_tiles]) return;
-    const int tile = chunk_tile(work.t_chunk0, n_tiles, w, &s_tile);
-    const TileGeom g = tile_geom(tile, tiles_x, W, H, work.ox, work.oy);
-    const size_t pix = (size_t)g.py * W + g.px;
-    const bool mine = g.inside && work.t_stop[pix] == (int32_t)w;
-    if (__syncthreads_count(mine) == 0) return;
-    const uint2 rg = ranges[tile];
-    const uint32_t a = rg.x + (w - work.t_chunk0[tile]) * kBwdChunk, b = min(rg.y, a + kBwdChunk);
-    const float4 sb = mine ? work.t_state[pix] : make_float4(0.f, 0.f, 0.f, 1.f);
-    Pixel px{sb.w, sb.x, sb.y, sb.z, mine ? work.t_slast[pix] : 0u, !mine, false};
-    composite_range<2>(sh, a, b, pval, rec, g.tx0, g.ty0, g.fpx, g.fpy, px);
-    if (mine) {
-        out[pix] = make_float4(px.r, px.g, px.b, 1.0f - px.T);
-        work.px_end[pix] = px.last;
-        work.px_fin[pix] = make_float4(px.r, px.g, px.b, px.T);
+        __syncwarp();  // the staging buffer is reused by the next chunk
     }
 }
 
 // Plan, part 1 (one thread per tile; meta zeroed before): tiles per list
 // length class (warp-aggregated atomics), and a slot plus
-// ceil((n - kBudget) / kChunk) consecutive chunks for every tile with more
-// than kBudget pairs.  Slot and chunk numbers depend on the order of the
+// ceil((n - budget) / kChunk) consecutive chunks for every tile with more
+// than budget pairs.  Slot and chunk numbers depend on the order of the
 // atomics; no result does (a tile's chunks are consecutive and merged in
 // order).
 __global__ void __launch_bounds__(256) k_blend_count(int n_tiles, const uint2 *__restrict__ ranges, BlendWork work) {
@@ -851,14 +945,14 @@ __global__ void __launch_bounds__(256) k_blend_count(int n_tiles, const uint2 *_
     if (cls >= 0 && lane == __ffs(peers) - 1) atomicAdd(work.meta + kBlendCountAt + cls, __popc(peers));
     if (t >= n_tiles) return;
     int slot = -1;
-    if (n > kBudget) {
-        const uint32_t nk = (n - kBudget + kChunk - 1) / kChunk;
+    if (n > work.budget) {
+        const uint32_t nk = (n - work.budget + kChunk - 1) / kChunk;
         slot = atomicAdd(work.meta + 0, 1);
         const uint32_t c0 = atomicAdd(reinterpret_cast<unsigned *>(work.meta + 1), nk);
         if (in_bounds((uint32_t)slot < work.max_slots && c0 + nk <= work.max_chunks, kChkSlot)) {
             work.cand_tile[slot] = t;
             work.cand_chunk0[slot] = c0;
-            work.cand_done[slot] = 1u;  // cleared by pass 1 unless every pixel is done
+            work.cand_done[slot] = 1u;  // cleared unless every pixel is closed
             for (uint32_t c = 0; c < nk; ++c) work.chunk_slot[c0 + c] = slot;
         } else {
             slot = -1;
@@ -905,46 +999,50 @@ static unsigned pp_grid() {
     return grid;
 }
 
-int launch_blend(int tiles_x, int tiles_y, int W, int H, const uint2 *ranges, const uint32_t *pval,
-                 const float4 *rec, float4 *out, const BlendWork &work, uint32_t n_pairs, cudaStream_t st) {
-    const int n = tiles_x * tiles_y;
-    if (n <= 0) return 0;
-    const size_t max_cand = blend_max_slots((size_t)n, n_pairs);
-    const size_t max_chunks = blend_max_chunks((size_t)n, n_pairs);
-    if (work.contrib) {
-        // statistics: every list composited in one pass
-        k_blend<1, kBlendThreads><<<n, kBlendThreads, 0, st>>>(tiles_x, W, H, ranges, pval, rec, out, work);
-        return 1;
-    }
-    if (work.px_end) {
-        // training forward: every list in parallel chunks, per-pixel state
-        // for the backward
-        k_train_counts<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, ranges, work.t_cnt);
-        const int sc = exclusive_scan(work.t_cnt, nullptr, work.t_chunk0, (uint32_t)n, work.t_scan, st);
-        const unsigned grid = (unsigned)train_max_chunks((size_t)n, n_pairs);
-        k_train_chunks<<<grid, kBlendThreads, 0, st>>>(tiles_x, W, H, ranges, pval, rec, work);
-        k_train_merge<<<n, kBlendThreads, 0, st>>>(tiles_x, W, H, ranges, out, work);
-        k_train_fix<<<grid, kBlendThreads, 0, st>>>(tiles_x, W, H, ranges, pval, rec, out, work);
-        return 4 + sc;
-    }
+// The plan's kernels: tile classes, slots and chunks, then the tile order.
+static int launch_plan(int n, const uint2 *ranges, const BlendWork &work, cudaStream_t st) {
     const unsigned tb = (unsigned)((n + 255) / 256);
     if (cudaMemsetAsync(work.meta, 0, kBlendMetaWords * sizeof(int32_t), st) != cudaSuccess) return -1;
     k_blend_count<<<tb, 256, 0, st>>>(n, ranges, work);
-    const unsigned grid = pp_grid();
-    k_blend_order<<<tb, 256, 0, st>>>(n, ranges, (int)grid, work);
-    // pass 1 of every tile: persistent CTAs, longest chains first
-    k_blend_pp<<<grid, kPpThreads, 0, st>>>(tiles_x, W, H, ranges, pval, rec, out, work);
-    const int launched = 3;
-    // no tile has pairs left after pass 1
-    if (n_pairs <= kBudget) return launched;
+    k_blend_order<<<tb, 256, 0, st>>>(n, ranges, (int)pp_grid(), work);
+    return 2;
+}
+
+// The split passes (nothing when no list is longer than the budget).
+template <bool kTrain>
+static int launch_split(int tiles_x, int W, int H, const uint2 *ranges, const uint32_t *pval, const float4 *rec,
+                        float4 *out, const BlendWork &work, cudaStream_t st) {
+    if (work.n_pairs <= work.budget) return 0;
     // chunk grids capped at kChunkGrid CTAs (grid-stride over the frame's
-    // chunks): a frame whose lists all end within the pass-1 budget does not
-    // pay for a worst-case grid of CTAs that return at once
-    const unsigned chunk_grid = (unsigned)std::min<size_t>(max_chunks, kChunkGrid);
-    k_blend_chunks<<<chunk_grid, kBlendThreads, 0, st>>>(tiles_x, W, H, ranges, pval, rec, work);
-    k_blend_merge<<<(unsigned)max_cand, kBlendThreads, 0, st>>>(tiles_x, W, H, ranges, out, work);
-    k_blend_fix<<<chunk_grid, kBlendThreads, 0, st>>>(tiles_x, W, H, ranges, pval, rec, out, work);
-    return launched + 3;
+    // chunks): a frame whose lists all end within the budget does not pay for
+    // a worst-case grid of CTAs that return at once
+    const unsigned chunk_grid = (unsigned)std::min<size_t>(work.max_chunks, kChunkGrid);
+    k_blend_chunks<kTrain><<<chunk_grid, kBlendThreads, 0, st>>>(tiles_x, W, H, ranges, pval, rec, work);
+    k_blend_merge<kTrain><<<work.max_slots, kBlendThreads, 0, st>>>(tiles_x, W, H, ranges, out, work);
+    k_blend_fix<kTrain><<<chunk_grid, kBlendThreads, 0, st>>>(tiles_x, W, H, ranges, pval, rec, out, work);
+    return 3;
+}
+
+int launch_blend(int tiles_x, int tiles_y, int W, int H, const uint2 *ranges, const uint32_t *pval,
+                 const float4 *rec, float4 *out, const BlendWork &work, cudaStream_t st) {
+    const int n = tiles_x * tiles_y;
+    if (n <= 0) return 0;
+    BlendWork w = work;
+    if (work.contrib || work.px_end) w.items = CS_BLEND_ITEMS_BLOCKS;  // tiles by decreasing list length class
+    int launched = launch_plan(n, ranges, w, st);
+    if (launched < 0) return -1;
+    if (work.contrib) {
+        // statistics: every list walked to its end
+        k_blend_walk<kStats><<<n, kBlendThreads, 0, st>>>(tiles_x, W, H, ranges, pval, rec, out, w);
+        return launched + 1;
+    }
+    if (work.px_end) {
+        k_blend_walk<kTraining><<<n, kBlendThreads, 0, st>>>(tiles_x, W, H, ranges, pval, rec, out, w);
+        return launched + 1 + launch_split<true>(tiles_x, W, H, ranges, pval, rec, out, w, st);
+    }
+    // pass 1 of every tile: persistent CTAs, longest chains first
+    k_blend_pp<<<pp_grid(), kPpThreads, 0, st>>>(tiles_x, W, H, ranges, pval, rec, out, w);
+    return launched + 1 + launch_split<false>(tiles_x, W, H, ranges, pval, rec, out, w, st);
 }
 
 CS_DEFINE_CHECK_READER(check_word_blend)

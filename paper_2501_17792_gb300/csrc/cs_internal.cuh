@@ -372,56 +372,47 @@ struct BlendWork {
     // when set: per splat, sum over pixels of its compositing weight
     // alpha * T (added to); lists are then composited in one pass
     float *contrib;
-    // when set (training forward, in chunks): per pixel, one past the index
-    // of its last composited pair and its final state (r, g, b, T).
-    // px_bnd: every pixel's state (r, g, b, T) before pair b of its tile's
-    // list, for every b = start + k kBwdChunk (k >= 1) up to the chunk in
-    // which the pixel stops, at px_bnd[(b / kBwdChunk) * 256 + pixel of the
-    // tile] (b / kBwdChunk is distinct for all such b of a frame: lists are
-    // disjoint)
+    // when set (training forward): per pixel, one past the index of its last
+    // composited pair and its final state (r, g, b, T).
+    // px_bnd: every open pixel's state (r, g, b, T) before pair b of its
+    // tile's list, for every b = start + k kBwdChunk (k >= 1) up to the chunk
+    // in which the pixel stops, at px_bnd[(b / kBwdChunk) * 256 + pixel of
+    // the tile] (b / kBwdChunk is distinct for all such b of a frame: lists
+    // are disjoint)
     uint32_t *px_end;
     float4 *px_fin;
     float4 *px_bnd;
-    // training forward in chunks of kBwdChunk pairs (numbered tile by tile):
-    // chunk counts per tile and their exclusive scan ([tiles + 1]), scan
-    // scratch; per chunk and pixel its composite from T = 1 (T negated when
-    // it met the stop rule) and one past its last composited pair (0: none);
-    // per image pixel the state before its stopping chunk, its last pair so
-    // far and that chunk (-1: none)
-    uint32_t *t_cnt, *t_chunk0, *t_scan;
-    float4 *t_part;
-    uint32_t *t_last;
-    float4 *t_state;
-    uint32_t *t_slast;
-    int32_t *t_stop;
+    // training, split lists: one past the last composited pair, per pass-2
+    // chunk and pixel (0: none) and per slot pixel before its stopping chunk
+    uint32_t *last, *slast;
     int32_t *pp_tile;     // [tiles]
     int32_t *chunk_slot;  // [chunks]: the slot of each pass-2 chunk
     int32_t ox, oy;       // window origin: pixel (i, j) has its centre at (ox + i + 0.5, oy + j + 0.5)
     int32_t items;        // pass-1 schedule: CS_BLEND_ITEMS_AUTO, _TILES or _BLOCKS
-    uint32_t n_pairs, max_slots, max_chunks;  // bounds of the checked debug build
+    uint32_t budget;      // pairs of a list before the split passes: kBlendBudget, kTrainBudget in training
+    uint32_t n_pairs, max_slots, max_chunks;  // pairs of the frame, slots and chunks its plan may need
 };
 constexpr int kBlendKeys = 64;     // schedule keys of pass 1 (see cs_blend.cu)
 constexpr int kBlendClasses = 24;  // list length classes: 0 empty, c: 2^(c-1) <= n < 2^c (last: n >= 2^22)
 constexpr int kBlendCountAt = 8, kBlendCursorAt = kBlendCountAt + kBlendClasses;
 constexpr int kBlendMetaWords = kBlendCursorAt + kBlendClasses;
 constexpr int kBlendBlockW = 8, kBlendBlockH = 4;  // pixels of one warp in a 16x16 tile
-constexpr uint32_t kBlendBudget = 32768;  // pairs composited by pass 1 per tile
+constexpr uint32_t kBlendBudget = 32768;  // pairs of a tile's list before the split passes
+constexpr uint32_t kTrainBudget = 8192;   // the same in training frames
 constexpr uint32_t kBlendChunk = 1024;   // pairs per pass-2 chunk
 constexpr uint32_t kBwdChunk = 1024;     // pairs per chunk of the compositing backward
 // boundary-state slots of a training frame of n_pairs pairs
 constexpr size_t bwd_boundary_slots(size_t n_pairs) { return n_pairs / kBwdChunk + 2; }
-// kBwdChunk-pair chunks of a frame of n_tiles tiles and n_pairs pairs, at most
-constexpr size_t train_max_chunks(size_t n_tiles, size_t n_pairs) { return n_pairs / kBwdChunk + n_tiles; }
-constexpr size_t blend_max_slots(size_t n_tiles, size_t n_pairs) {
-    return n_tiles < n_pairs / kBlendBudget + 1 ? n_tiles : n_pairs / kBlendBudget + 1;
+constexpr size_t blend_max_slots(size_t n_tiles, size_t n_pairs, size_t budget = kBlendBudget) {
+    return n_tiles < n_pairs / budget + 1 ? n_tiles : n_pairs / budget + 1;
 }
-constexpr size_t blend_max_chunks(size_t n_tiles, size_t n_pairs) {
-    return n_pairs / kBlendChunk + blend_max_slots(n_tiles, n_pairs) + 1;
+constexpr size_t blend_max_chunks(size_t n_tiles, size_t n_pairs, size_t budget = kBlendBudget) {
+    return n_pairs / kBlendChunk + blend_max_slots(n_tiles, n_pairs, budget) + 1;
 }
 // Returns the kernels launched, or -1 when the plan's counters could not be
 // cleared (the CUDA error is then cudaGetLastError's).
 int launch_blend(int tiles_x, int tiles_y, int W, int H, const uint2 *ranges, const uint32_t *pval,
-                 const float4 *rec, float4 *out, const BlendWork &work, uint32_t n_pairs, cudaStream_t st);
+                 const float4 *rec, float4 *out, const BlendWork &work, cudaStream_t st);
 
 }  // namespace cs
 
