@@ -90,7 +90,7 @@ struct cs_ctx {
     DevBuf<uint32_t> px_end, bwd_cnt, bwd_chunk0, bwd_scratch;
     DevBuf<float4> px_fin, px_bnd;  // training: final state per pixel, states at the backward chunk boundaries
     DevBuf<uint32_t> t_last, t_slast;  // training, split lists: last pair per chunk pixel and slot pixel
-    DevBuf<float> g_cov, g_B, g_dummy;
+    DevBuf<float> g_acc, g_B, g_dummy;
     DevBuf<float4> dsplat;
     bool train_valid = false;
     CamParams train_cp{};
@@ -453,7 +453,7 @@ void cs_destroy(cs_ctx *ctx) {
     release(ctx->ptile2); release(ctx->img); release(ctx->contrib_s); release(ctx->dbg_rec);
     release(ctx->px_end); release(ctx->px_fin); release(ctx->px_bnd); release(ctx->bwd_cnt); release(ctx->bwd_chunk0);
     release(ctx->bwd_scratch); release(ctx->t_last);
-    release(ctx->t_slast); release(ctx->dsplat); release(ctx->g_cov); release(ctx->g_B);
+    release(ctx->t_slast); release(ctx->dsplat); release(ctx->g_acc); release(ctx->g_B);
     release(ctx->g_dummy);
     release(ctx->bw_slot); release(ctx->bw_tile); release(ctx->bw_meta); release(ctx->bw_stop); release(ctx->bw_pp); release(ctx->bw_cslot); release(ctx->bw_chunk0);
     release(ctx->bw_done); release(ctx->bw_state); release(ctx->bw_part);
@@ -1129,12 +1129,12 @@ int cs_backward(cs_ctx *ctx, const float *dl_drgba, const cs_grads *grads) {
     CS_TRY(ensure(ctx, ctx->bwd_cnt, nt, "backward chunk counts"));
     CS_TRY(ensure(ctx, ctx->bwd_chunk0, nt + 1, "backward chunk offsets"));
     CS_TRY(ensure(ctx, ctx->bwd_scratch, scan_scratch_words(nt), "backward scan scratch"));
-    CS_TRY(ensure(ctx, ctx->g_cov, G * 6, "covariance gradients"));
+    CS_TRY(ensure(ctx, ctx->g_acc, G * 12, "Gaussian gradients"));
     CS_TRY(ensure(ctx, ctx->g_B, I * kJoints * 12, "skinning-transform gradients"));
     // destinations the caller does not want go to one scratch buffer
     CS_TRY(ensure(ctx, ctx->g_dummy, std::max(G * 48, I * kJoints * 3), "gradient scratch"));
     CS_CUDA(cudaMemsetAsync(ctx->dsplat.p, 0, S * 3 * sizeof(float4), st));
-    CS_CUDA(cudaMemsetAsync(ctx->g_cov.p, 0, G * 6 * sizeof(float), st));
+    CS_CUDA(cudaMemsetAsync(ctx->g_acc.p, 0, G * 12 * sizeof(float), st));
     CS_CUDA(cudaMemsetAsync(ctx->g_B.p, 0, I * kJoints * 12 * sizeof(float), st));
     BackwardArgs a{};
     a.tiles_x = cp.tiles_x;
@@ -1169,12 +1169,13 @@ int cs_backward(cs_ctx *ctx, const float *dl_drgba, const cs_grads *grads) {
     a.sh_frame = ctx->sh_frame;
     float *dummy = ctx->g_dummy.p;
     a.g_mean = grads->means ? grads->means : dummy;
-    a.g_cov = ctx->g_cov.p;
+    a.g_acc = ctx->g_acc.p;
     a.g_opacity = grads->opacity ? grads->opacity : dummy;
     a.g_sh = grads->sh ? grads->sh : dummy;
     a.g_B = ctx->g_B.p;
     a.n_inst = ctx->n_inst;
     a.n_tpl = ctx->n_tpl;
+    a.max_depth = ctx->max_depth;
     a.tid = ctx->tid.p;
     a.pose = ctx->pose.p;
     a.g_pose = grads->pose ? grads->pose : dummy;
@@ -1277,7 +1278,7 @@ int cs_memory_stats(cs_ctx *ctx, cs_memory_stats_t *out) {
                  bytes_of(ctx->px_end) + bytes_of(ctx->px_fin) + bytes_of(ctx->px_bnd) + bytes_of(ctx->bwd_cnt) +
                  bytes_of(ctx->bwd_chunk0) + bytes_of(ctx->bwd_scratch) + bytes_of(ctx->t_last) +
                  bytes_of(ctx->t_slast) + bytes_of(ctx->dsplat) +
-                 bytes_of(ctx->g_cov) +
+                 bytes_of(ctx->g_acc) +
                  bytes_of(ctx->g_B) + bytes_of(ctx->g_dummy);
     out->template_bytes = tb;
     out->instance_bytes = ib;

@@ -433,7 +433,9 @@ struct BackwardArgs {
     uint32_t *chunk0;
     uint32_t *scan_scratch;
     const float4 *dl_drgba;
-    float4 *dsplat;  // [S][3]: du, dv, dA, dB | dC, do, dr, dg | db, -, -, -
+    // [S][3], zeroed: per splat, with G = dL/dalpha alpha summed over pixels,
+    // G, G dx, G dy, G dx^2 | G dx dy, G dy^2, dr, dg | db, -, -, -
+    float4 *dsplat;
     int proj_blocks;
     const Group *groups;
     int n_groups;
@@ -444,8 +446,9 @@ struct BackwardArgs {
     CamParams cam;
     LodParams lod;
     int skin_mode, sh_frame;
-    float *g_mean, *g_cov, *g_opacity, *g_sh, *g_B;
-    int n_inst, n_tpl;
+    float *g_acc;  // [n_gauss][12], zeroed: mean, opacity, canonical covariance (see cs_backward.cu)
+    float *g_mean, *g_opacity, *g_sh, *g_B;
+    int n_inst, n_tpl, max_depth;
     const int32_t *tid;
     const float *pose;
     float *g_pose;
