@@ -772,8 +772,8 @@ __device__ __forceinline__ void project_chunk(
     bin[s] = live ? bword : 0u;
 }
 
-// Projection CTAs: kChunks consecutive virtual blocks each (8 with FP32
-// storage), a virtual block being 256 Gaussians of one visible instance
+// Projection CTAs: kChunks consecutive virtual blocks each (launch_project
+// chooses), a virtual block being 256 Gaussians of one visible instance
 // (cull_group numbers them: Group::block0).  Consecutive virtual blocks
 // mostly belong to one instance, whose transforms are then staged once.  kChunks = 1 for BF16 storage (its
 // tensor-core blend reuses shared memory between barriers).
@@ -865,7 +865,15 @@ __global__ void __launch_bounds__(kProjThreads, 5) k_project(
     }
 }
 
-constexpr int kProjChunksFp32 = 8;
+// Virtual blocks per CTA.  A CTA's chunks run one after the other (one round
+// of load latency each), so a frame that fits the device in a few waves takes
+// one per CTA; larger frames take kProjChunks, which stage an instance's
+// transforms once for several chunks and launch fewer CTAs.
+// One chunk against eight: 16,384 Gaussians at 256x256 234 -> 222 us a frame,
+// 202,738 at 1280x720 402 -> 385 us, 100 x 12,661 505 -> 503 us (5,000
+// blocks); four against eight are equal from 16,384 blocks up.
+constexpr int kProjChunks = 4;
+constexpr int kProjOneChunkBlocks = 8192;
 
 int launch_project(int n_blocks, const Group *groups, const Group *groups_host, int n_groups,
                    const TemplateInfo *tpl_host, const int32_t *vis, const float *B, const float *V,
@@ -894,9 +902,13 @@ int launch_project(int n_blocks, const Group *groups, const Group *groups_host, 
         k_project<kStoreBf16, 1><<<n_blocks, kProjThreads, 0, st>>>(groups, n_groups, n_blocks, vis, B, V, root, ta,
                                                                    tpls, cam, lod, skin_mode, sh_frame, rec,
                                                                    key, bin, pg);
+    } else if (n_blocks <= kProjOneChunkBlocks) {
+        k_project<kStoreFp32, 1><<<n_blocks, kProjThreads, 0, st>>>(groups, n_groups, n_blocks, vis, B, V, root, ta,
+                                                                    tpls, cam, lod, skin_mode, sh_frame, rec,
+                                                                    key, bin, pg);
     } else {
-        const int grid = (n_blocks + kProjChunksFp32 - 1) / kProjChunksFp32;
-        k_project<kStoreFp32, kProjChunksFp32><<<grid, kProjThreads, 0, st>>>(
+        const int grid = (n_blocks + kProjChunks - 1) / kProjChunks;
+        k_project<kStoreFp32, kProjChunks><<<grid, kProjThreads, 0, st>>>(
             groups, n_groups, n_blocks, vis, B, V, root, ta, tpls, cam, lod, skin_mode, sh_frame, rec, key,
             bin, pg);
     }
