@@ -869,8 +869,8 @@ __global__ void __launch_bounds__(kProjThreads, 5) k_project(
 // of load latency each), so a frame that fits the device in a few waves takes
 // one per CTA; larger frames take kProjChunks, which stage an instance's
 // transforms once for several chunks and launch fewer CTAs.
-// One chunk against eight: 16,384 Gaussians at 256x256 234 -> 222 us a frame,
-// 202,738 at 1280x720 402 -> 385 us, 100 x 12,661 505 -> 503 us (5,000
+// One chunk against eight: 16,384 Gaussians at 256x256 232 -> 218 us a frame,
+// 202,738 at 1280x720 405 -> 382 us, 100 x 12,661 509 -> 496 us (5,000
 // blocks); four against eight are equal from 16,384 blocks up.
 constexpr int kProjChunks = 4;
 constexpr int kProjOneChunkBlocks = 8192;
