@@ -1002,7 +1002,6 @@ static unsigned pp_grid() {
 // The plan's kernels: tile classes, slots and chunks, then the tile order.
 static int launch_plan(int n, const uint2 *ranges, const BlendWork &work, cudaStream_t st) {
     const unsigned tb = (unsigned)((n + 255) / 256);
-    if (cudaMemsetAsync(work.meta, 0, kBlendMetaWords * sizeof(int32_t), st) != cudaSuccess) return -1;
     k_blend_count<<<tb, 256, 0, st>>>(n, ranges, work);
     k_blend_order<<<tb, 256, 0, st>>>(n, ranges, (int)pp_grid(), work);
     return 2;
@@ -1030,7 +1029,6 @@ int launch_blend(int tiles_x, int tiles_y, int W, int H, const uint2 *ranges, co
     BlendWork w = work;
     if (work.contrib || work.px_end) w.items = CS_BLEND_ITEMS_BLOCKS;  // tiles by decreasing list length class
     int launched = launch_plan(n, ranges, w, st);
-    if (launched < 0) return -1;
     if (work.contrib) {
         // statistics: every list walked to its end
         k_blend_walk<kStats><<<n, kBlendThreads, 0, st>>>(tiles_x, W, H, ranges, pval, rec, out, w);

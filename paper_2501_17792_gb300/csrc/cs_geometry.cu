@@ -42,7 +42,9 @@ __device__ __forceinline__ void rodrigues(float x, float y, float z, float R[9])
 __global__ void __launch_bounds__(256) k_fk(int n_inst, int n_tpl, const int32_t *__restrict__ tid,
                                             const float *__restrict__ pose,
                                             const TemplateInfo *__restrict__ tpls, int max_depth,
-                                            float *__restrict__ B) {
+                                            float *__restrict__ B, int32_t *__restrict__ cull_tot, int n_tot) {
+    if (blockIdx.x == 0)
+        for (int i = threadIdx.x; i < n_tot; i += blockDim.x) cull_tot[i] = 0;
     const int inst = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (inst >= n_inst) return;  // uniform per warp
@@ -97,10 +99,29 @@ __global__ void __launch_bounds__(256) k_fk(int n_inst, int n_tpl, const int32_t
 }
 
 int launch_fk(int n_inst, int n_tpl, const int32_t *tid, const float *pose, const TemplateInfo *tpls,
-              int max_depth, float *B, cudaStream_t st) {
+              int max_depth, float *B, int32_t *cull_scratch, cudaStream_t st) {
     if (n_inst <= 0) return 0;
     int blocks = (n_inst + 7) / 8;
-    k_fk<<<blocks, 256, 0, st>>>(n_inst, n_tpl, tid, pose, tpls, max_depth, B);
+    k_fk<<<blocks, 256, 0, st>>>(n_inst, n_tpl, tid, pose, tpls, max_depth, B, cull_scratch, kMaxGroups + 3);
+    return 1;
+}
+
+__global__ void __launch_bounds__(256) k_copy_instances(int n, const int32_t *__restrict__ tid,
+                                                        const float *__restrict__ root,
+                                                        const float *__restrict__ pose, int32_t *__restrict__ tid_out,
+                                                        float *__restrict__ root_out, float *__restrict__ pose_out) {
+    const int stride = gridDim.x * blockDim.x, i0 = blockIdx.x * blockDim.x + threadIdx.x;
+    for (int i = i0; i < n * kJoints * 3; i += stride) {
+        pose_out[i] = pose[i];
+        if (i < n * 12) root_out[i] = root[i];
+        if (i < n) tid_out[i] = tid[i];
+    }
+}
+
+int launch_copy_instances(int n, const int32_t *tid, const float *root, const float *pose, int32_t *tid_out,
+                          float *root_out, float *pose_out, cudaStream_t st) {
+    const int blocks = (n * kJoints * 3 + 1023) / 1024;  // four floats a thread
+    k_copy_instances<<<blocks, 256, 0, st>>>(n, tid, root, pose, tid_out, root_out, pose_out);
     return 1;
 }
 
@@ -114,7 +135,7 @@ int launch_fk(int n_inst, int n_tpl, const int32_t *tid, const float *pose, cons
 
 constexpr int kCullThreads = 1024;
 constexpr uint8_t kHidden = 255;
-// frame totals in the cull scratch (zeroed before the launch): group counts,
+// frame totals in the cull scratch (zeroed by k_fk): group counts,
 // then the inverted bits of the lowest depth bound, the highest, the ticket
 constexpr int kCullZloInv = kMaxGroups, kCullZhi = kMaxGroups + 1, kCullTicket = kMaxGroups + 2;
 
@@ -122,8 +143,8 @@ __global__ void __launch_bounds__(kCullThreads) k_cull_group(
     int n_inst, int n_tpl, const int32_t *__restrict__ tid, const float *__restrict__ root,
     const TemplateInfo *__restrict__ tpls, CamParams cam, LodParams lod, int do_cull,
     float *__restrict__ V, float *__restrict__ Cloc, int32_t *__restrict__ vis,
-    Group *__restrict__ groups, int32_t *__restrict__ meta, int32_t *__restrict__ tot,
-    uint8_t *__restrict__ grp) {
+    Group *__restrict__ groups, int32_t *__restrict__ meta, int32_t *host_meta, Group *host_groups, uint32_t seq,
+    int32_t *__restrict__ tot, uint8_t *__restrict__ grp) {
     __shared__ int32_t gcount[kMaxGroups];
     __shared__ int32_t gslot[kMaxGroups];
     __shared__ int32_t wcount[kCullThreads / 32][kMaxGroups];  // per warp and group
@@ -273,6 +294,14 @@ __global__ void __launch_bounds__(kCullThreads) k_cull_group(
         meta[kMetaZhi] = (int32_t)zhi_bits;
     }
     __syncthreads();
+    // what the host waits for, ahead of the placement: the groups, the counts,
+    // then the frame's sequence number
+    for (int w = threadIdx.x; w < meta[kMetaGroups] * (int)(sizeof(Group) / 4); w += kCullThreads)
+        reinterpret_cast<int32_t *>(host_groups)[w] = reinterpret_cast<const int32_t *>(groups)[w];
+    if (threadIdx.x < kMetaSeq) host_meta[threadIdx.x] = meta[threadIdx.x];
+    __threadfence_system();
+    __syncthreads();
+    if (threadIdx.x == 0) *reinterpret_cast<volatile uint32_t *>(host_meta + kMetaSeq) = seq;
     // stable placement, one round of kCullThreads instances at a time: an
     // instance goes to its group's slot plus the instances of its group in
     // earlier rounds (gslot runs on), in earlier warps of the round (a scan
@@ -307,11 +336,11 @@ size_t cull_scratch_words(size_t n_inst) { return kMaxGroups + 3 + (n_inst + 3) 
 int launch_cull_group(int n_inst, int n_tpl, const int32_t *tid, const float *root,
                        const TemplateInfo *tpls, const CamParams &cam, const LodParams &lod,
                        int do_cull, float *V, float *Cloc, int32_t *vis, Group *groups,
-                       int32_t *meta, int32_t *scratch, cudaStream_t st) {
-    if (cudaMemsetAsync(scratch, 0, (kMaxGroups + 3) * sizeof(int32_t), st) != cudaSuccess) return -1;
+                       int32_t *meta, int32_t *host_meta, Group *host_groups, uint32_t seq, int32_t *scratch,
+                       cudaStream_t st) {
     const unsigned blocks = (unsigned)((n_inst + kCullThreads - 1) / kCullThreads);
     k_cull_group<<<blocks > 0 ? blocks : 1u, kCullThreads, 0, st>>>(
-        n_inst, n_tpl, tid, root, tpls, cam, lod, do_cull, V, Cloc, vis, groups, meta, scratch,
+        n_inst, n_tpl, tid, root, tpls, cam, lod, do_cull, V, Cloc, vis, groups, meta, host_meta, host_groups, seq, scratch,
         reinterpret_cast<uint8_t *>(scratch + kMaxGroups + 3));
     return 1;
 }

@@ -266,6 +266,7 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t *t
 enum MetaIndex {
     kMetaVisible = 0, kMetaGroups = 1, kMetaSplats = 2, kMetaLevel0 = 3, kMetaBlocks = 7,
     kMetaZlo = 8, kMetaZhi = 9,  // float bits of a lower / upper bound of every live splat depth
+    kMetaSeq = 10,  // host copy: the sequence number of the frame the words belong to
     kMetaWords = 12
 };
 
@@ -285,17 +286,22 @@ int launch_contrib_to_template(int n_splats, const Group *groups, int n_groups, 
                                const uint32_t *lod_idx, const float *contrib_splat, float *contrib_tmpl,
                                cudaStream_t st);
 // ---- geometry (cs_geometry.cu) ----
+// Copies n instances' template ids, roots and poses (device arrays) in one launch.
+int launch_copy_instances(int n, const int32_t *tid, const float *root, const float *pose, int32_t *tid_out,
+                          float *root_out, float *pose_out, cudaStream_t st);
+// Also clears the cull's frame totals (cull_scratch).
 int launch_fk(int n_inst, int n_tpl, const int32_t *tid, const float *pose, const TemplateInfo *tpls,
-              int max_depth, float *B, cudaStream_t st);
+              int max_depth, float *B, int32_t *cull_scratch, cudaStream_t st);
 // Cull scratch of n instances (frame totals, then a group byte per
 // instance), in 4-byte words.
 size_t cull_scratch_words(size_t n_inst);
-// Returns the kernels launched, or -1 when the scratch could not be cleared
-// (the CUDA error is then cudaGetLastError's).
+// Runs after launch_fk.  The counts and groups also go to host_meta and
+// host_groups (pinned host memory), then seq to host_meta[kMetaSeq].
 int launch_cull_group(int n_inst, int n_tpl, const int32_t *tid, const float *root,
                        const TemplateInfo *tpls, const CamParams &cam, const LodParams &lod,
                        int do_cull, float *V, float *Cloc, int32_t *vis, Group *groups,
-                       int32_t *meta, int32_t *scratch, cudaStream_t st);
+                       int32_t *meta, int32_t *host_meta, Group *host_groups, uint32_t seq, int32_t *scratch,
+                       cudaStream_t st);
 int launch_project(int n_blocks, const Group *groups, const Group *groups_host, int n_groups,
                    const TemplateInfo *tpl_host, const int32_t *vis, const float *B, const float *V,
                    const float *root, const TemplateArrays &ta, const TemplateInfo *tpls,
@@ -335,12 +341,14 @@ int radix_sort_u16(uint16_t *k0, uint32_t *v0, uint16_t *k1, uint32_t *v1, uint3
 // bin_scan_sums writes the per-block sums of the sorted bin words' pair
 // counts, exclusively scanned, to sums[0 .. nb) and the total to sums[nb]
 // (nb = bin_scan_blocks(n)); launch_emit_pairs_scan then writes every
-// splat's pairs (the scan's down-sweep fused into the emission).
+// splat's pairs (the scan's down-sweep fused into the emission) and clears
+// the tile ranges and the compositing's plan counters for the kernels after it.
 size_t bin_scan_blocks(size_t n);
-int bin_scan_sums(const uint32_t *bins, uint32_t n, uint32_t *sums, cudaStream_t st);
+// host (pinned host memory) receives the total and then seq in host[2].
+int bin_scan_sums(const uint32_t *bins, uint32_t n, uint32_t *sums, uint32_t *host, uint32_t seq, cudaStream_t st);
 int launch_emit_pairs_scan(uint32_t n_splats, const uint32_t *order, const uint32_t *bins_sorted,
                            const uint32_t *sums, const float4 *rec, int tiles_x, uint32_t n_tiles, uint16_t *ptile,
-                           uint32_t *pval, cudaStream_t st);
+                           uint32_t *pval, uint2 *ranges, int32_t *blend_meta, cudaStream_t st);
 int launch_emit_pairs(uint32_t n_splats, const uint32_t *order, const uint32_t *bins_sorted,
                       const uint32_t *pair_off, const float4 *rec, int tiles_x, uint32_t n_tiles, uint16_t *ptile,
                       uint32_t *pval, cudaStream_t st);
@@ -409,8 +417,7 @@ constexpr size_t blend_max_slots(size_t n_tiles, size_t n_pairs, size_t budget =
 constexpr size_t blend_max_chunks(size_t n_tiles, size_t n_pairs, size_t budget = kBlendBudget) {
     return n_pairs / kBlendChunk + blend_max_slots(n_tiles, n_pairs, budget) + 1;
 }
-// Returns the kernels launched, or -1 when the plan's counters could not be
-// cleared (the CUDA error is then cudaGetLastError's).
+// work.meta must be zero.  Returns the kernels launched.
 int launch_blend(int tiles_x, int tiles_y, int W, int H, const uint2 *ranges, const uint32_t *pval,
                  const float4 *rec, float4 *out, const BlendWork &work, cudaStream_t st);
 

@@ -49,8 +49,10 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const uint32_t *__
     if (threadIdx.x == 0) sums[blockIdx.x] = total;
 }
 
-// One block: exclusive scan of the tile sums in place, total at sums[nb].
-__global__ void __launch_bounds__(kScanThreads) k_scan_spine(uint32_t *__restrict__ sums, uint32_t nb) {
+// One block: exclusive scan of the tile sums in place, total at sums[nb]
+// (and, when set, at host[0] in pinned host memory, then seq at host[2]).
+__global__ void __launch_bounds__(kScanThreads) k_scan_spine(uint32_t *__restrict__ sums, uint32_t nb, uint32_t *host,
+                                                             uint32_t seq) {
     __shared__ uint32_t total;
     uint32_t carry = 0;
     for (uint32_t base = 0; base < nb; base += kScanThreads) {
@@ -62,7 +64,14 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_spine(uint32_t *__restric
         carry += total;
         __syncthreads();
     }
-    if (threadIdx.x == 0) sums[nb] = carry;
+    if (threadIdx.x == 0) {
+        sums[nb] = carry;
+        if (host) {
+            host[0] = carry;
+            __threadfence_system();
+            *reinterpret_cast<volatile uint32_t *>(host + 2) = seq;
+        }
+    }
 }
 
 template <int MODE>
@@ -97,7 +106,7 @@ static int scan_impl(const uint32_t *in, uint32_t *out, uint32_t n, uint32_t *sc
     }
     const uint32_t nb = (n + kScanTile - 1) / kScanTile;
     k_scan_reduce<MODE><<<nb, kScanThreads, 0, st>>>(in, n, scratch);
-    k_scan_spine<<<1, kScanThreads, 0, st>>>(scratch, nb);
+    k_scan_spine<<<1, kScanThreads, 0, st>>>(scratch, nb, nullptr, 0u);
     k_scan_down<MODE><<<nb, kScanThreads, 0, st>>>(in, n, scratch, nb, out);
     return 3;
 }
@@ -463,8 +472,13 @@ __global__ void __launch_bounds__(kScanThreads) k_emit_pairs_scan(uint32_t n, co
                                                                  const uint32_t *__restrict__ sums,
                                                                  const float4 *__restrict__ rec, int tiles_x,
                                                                  uint32_t n_tiles, uint16_t *__restrict__ ptile,
-                                                                 uint32_t *__restrict__ pval) {
+                                                                 uint32_t *__restrict__ pval,
+                                                                 uint2 *__restrict__ ranges,
+                                                                 int32_t *__restrict__ blend_meta) {
     __shared__ uint32_t total, n_large;
+    for (uint32_t k = blockIdx.x * kScanThreads + threadIdx.x; k < n_tiles; k += gridDim.x * kScanThreads)
+        ranges[k] = make_uint2(0u, 0u);
+    if (blockIdx.x == 0 && threadIdx.x < kBlendMetaWords) blend_meta[threadIdx.x] = 0;
     const uint32_t n_pairs = CS_CHECKS ? sums[gridDim.x] : 0xFFFFFFFFu;  // the scan's total
     __shared__ uint4 s_large[kScanThreads];  // splat id, first pair, tile x0 | y0 << 16, tiles per row
     __shared__ uint32_t s_cnt[kScanThreads];  // its pairs
@@ -512,20 +526,20 @@ __global__ void __launch_bounds__(kScanThreads) k_emit_pairs_scan(uint32_t n, co
 
 size_t bin_scan_blocks(size_t n) { return (n + kScanTile - 1) / kScanTile; }
 
-int bin_scan_sums(const uint32_t *bins, uint32_t n, uint32_t *sums, cudaStream_t st) {
+int bin_scan_sums(const uint32_t *bins, uint32_t n, uint32_t *sums, uint32_t *host, uint32_t seq, cudaStream_t st) {
     if (n == 0) return 0;
     const uint32_t nb = (uint32_t)bin_scan_blocks(n);
     k_scan_reduce<1><<<nb, kScanThreads, 0, st>>>(bins, n, sums);
-    k_scan_spine<<<1, kScanThreads, 0, st>>>(sums, nb);
+    k_scan_spine<<<1, kScanThreads, 0, st>>>(sums, nb, host, seq);
     return 2;
 }
 
 int launch_emit_pairs_scan(uint32_t n_splats, const uint32_t *order, const uint32_t *bins_sorted,
                            const uint32_t *sums, const float4 *rec, int tiles_x, uint32_t n_tiles, uint16_t *ptile,
-                           uint32_t *pval, cudaStream_t st) {
+                           uint32_t *pval, uint2 *ranges, int32_t *blend_meta, cudaStream_t st) {
     if (n_splats == 0) return 0;
     k_emit_pairs_scan<<<(uint32_t)bin_scan_blocks(n_splats), kScanThreads, 0, st>>>(
-        n_splats, order, bins_sorted, sums, rec, tiles_x, n_tiles, ptile, pval);
+        n_splats, order, bins_sorted, sums, rec, tiles_x, n_tiles, ptile, pval, ranges, blend_meta);
     return 1;
 }
 

@@ -80,3 +80,27 @@ def test_gradients_into_an_sh_array_off_the_16_byte_grid(sh_degree):
     assert torch.allclose(buf[1:-1], want, rtol=1e-4, atol=1e-5 * float(want.abs().max()))
     assert float(buf[0]) == 0.0 and float(buf[-1]) == 0.0 and float(want.abs().max()) > 0.0
     r.close()
+
+
+def test_counts_of_a_new_context_after_contexts_of_one_frame():
+    """The host polls a frame's counts in pinned memory that an earlier
+    context may have used: contexts that render one frame of different sizes
+    and go, then one of the first size again, all equal to a context that
+    stays."""
+    from paper_2501_17792_gb300 import binding
+    from paper_2501_17792_gb300 import scene as S
+    small, large = (S.crowd(n_templates=1, n_gauss=n, sh_degree=0, cols=c, rows=4, width=96, height=64)
+                    for n, c in ((300, 3), (5000, 6)))
+    for on_device in (False, True):
+        want = {}
+        for k in range(6):
+            sc = (small, large)[k % 2]
+            r = binding.Renderer(device=0)
+            r.upload_templates(sc.templates)
+            r.set_lod(sc.lod)
+            inst = [sc.instances.template_id, sc.instances.root, sc.instances.pose]
+            r.set_instances(*([torch.from_numpy(a).cuda() for a in inst] if on_device else inst))
+            img = r.render(sc.camera).clone()
+            r.close()
+            assert torch.equal(img, want.setdefault(k % 2, img))
+            assert float(img[..., 3].max()) > 0.5
