@@ -37,16 +37,22 @@ constexpr int kP = CS_MLP_PARAMS;   // 7361
 constexpr int oW1 = 0, oB1 = oW1 + kIn * kH, oW2 = oB1 + kH, oB2 = oW2 + kH * kH, oW3 = oB2 + kH, oB3 = oW3 + kH;
 static_assert(oB3 + 1 == kP, "parameter layout");
 
-constexpr int kWarps = 8, kThreads = 32 * kWarps, kTile = 16 * kWarps;  // 128 rows per CTA tile
-// shared-memory leading dimensions (bf16 elements), padded so that the 32
-// lanes of a fragment load hit 32 different banks
+// Warps of a CTA, 16 rows of its tile each.  Training: 12 warps of at most 168
+// registers, one CTA per SM, which hold a thread's 72 gradient sums; the
+// forward pass alone needs half of them.
+__host__ __device__ constexpr int mlp_warps(bool train) { return train ? 12 : 8; }
+__host__ __device__ constexpr int mlp_tile(bool train) { return 16 * mlp_warps(train); }
+// shared-memory leading dimensions (bf16 elements): 28 and 36 words, so that
+// the eight 16-byte rows of an ldmatrix and the 32 words of a fragment store
+// fall in different banks
 constexpr int kLdW1 = 56;   // W1^T  [64 hidden][48 in]
 constexpr int kLdW2 = 72;   // W2^T and W2 [64][64]
-constexpr int kLdT = kTile + 8;  // transposed activations [feature][row]
+constexpr int kLdX = 56;    // activations by row: inputs [row][48],
+constexpr int kLdA = 72;    // hidden units [row][64]
 
 constexpr size_t kW1Elems = (size_t)kH * kLdW1, kW2Elems = (size_t)kH * kLdW2;
 constexpr size_t kSmemWeights = (kW1Elems + 2 * kW2Elems) * 2 + (3 * kH + 4) * 4;
-constexpr size_t kSmemTrain = kSmemWeights + (size_t)(kIn + 3 * kH) * kLdT * 2 + (3 * kWarps * kH + 2 * kWarps) * 4;
+constexpr size_t kSmemTrain = kSmemWeights + (size_t)mlp_tile(true) * (kLdX + 3 * kLdA) * 2 + (3 * kH + 2) * mlp_warps(true) * 4;
 
 struct Weights {
     const __nv_bfloat16 *w1t;  // [64][kLdW1]: w1t[n][k] = bf16(W1[k][n])
@@ -56,7 +62,7 @@ struct Weights {
 };
 
 __device__ __forceinline__ void mma16816(float d[4], const uint32_t a[4], uint32_t b0, uint32_t b1) {
-    asm volatile(
+    asm(
         "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
         "{%0,%1,%2,%3};\n"
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
@@ -65,34 +71,93 @@ __device__ __forceinline__ void mma16816(float d[4], const uint32_t a[4], uint32
 
 __device__ __forceinline__ uint32_t bits16(__nv_bfloat16 v) { return (uint32_t)__bfloat16_as_ushort(v); }
 __device__ __forceinline__ uint32_t pack2(__nv_bfloat16 lo, __nv_bfloat16 hi) { return bits16(lo) | (bits16(hi) << 16); }
-__device__ __forceinline__ uint32_t ld32(const __nv_bfloat16 *p) { return *reinterpret_cast<const uint32_t *>(p); }
+__device__ __forceinline__ void st32(__nv_bfloat16 *p, uint32_t v) { *reinterpret_cast<uint32_t *>(p) = v; }
 
-// Input x[row][c]: features for c < 32, one-hot band for 32 <= c < 36, zero above.
-__device__ __forceinline__ float2 input_pair(const float *__restrict__ feat, int band, bool valid, int row, int c) {
-    if (!valid) return make_float2(0.f, 0.f);
-    if (c < kFeat) return __ldg(reinterpret_cast<const float2 *>(feat + (size_t)row * kFeat + c));
-    const int b = c - kFeat;
-    return make_float2(b == band ? 1.f : 0.f, b + 1 == band ? 1.f : 0.f);
+// Four 8x8 bf16 matrices (rows of 16 bytes at the lanes' addresses, lanes 8 i
+// to 8 i + 7 giving matrix i); trans: each transposed.
+__device__ __forceinline__ void ldsm4(uint32_t r[4], const __nv_bfloat16 *p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"((uint32_t)__cvta_generic_to_shared(p))
+                 : "memory");
+}
+__device__ __forceinline__ void ldsm4t(uint32_t r[4], const __nv_bfloat16 *p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"((uint32_t)__cvta_generic_to_shared(p))
+                 : "memory");
 }
 
+constexpr int kChains = 2;  // independent products in flight: column tiles computed at a time (4: 545 us against 541)
+
+// d[i] += a (16 rows x 64) times column tile i of a weight matrix in shared
+// memory; wp: row mr of the first tile, column 8 mi.
+__device__ __forceinline__ void mma_chains(float (&d)[kChains][4], const uint32_t (&a)[4][4], const __nv_bfloat16 *wp) {
+#pragma unroll
+    for (int kk = 0; kk < 4; kk += 2) {
+        uint32_t b[kChains][4];
+#pragma unroll
+        for (int i = 0; i < kChains; ++i) ldsm4(b[i], wp + 8 * i * kLdW2 + 16 * kk);
+#pragma unroll
+        for (int i = 0; i < kChains; ++i) mma16816(d[i], a[kk], b[i][0], b[i][1]);
+#pragma unroll
+        for (int i = 0; i < kChains; ++i) mma16816(d[i], a[kk + 1], b[i][2], b[i][3]);
+    }
+}
+
+// What a lane reads of its rows g and g + 8: features 8 i + 2 q and the next
+// (i = 0 to 3), the band (-1: none, an all-zero one-hot) and the target.
+struct RowInputs {
+    float2 x[2][4];
+    int band[2];
+    float target[2];
+};
+
 template <bool kTrain>
-__global__ void __launch_bounds__(kThreads, 1) k_mlp(int64_t n, int n_tiles, const float *__restrict__ feat,
-                                                     const int32_t *__restrict__ band,
-                                                     const float *__restrict__ target, Weights W, float inv_n,
-                                                     float *__restrict__ score, float *__restrict__ partial) {
+__device__ __forceinline__ void load_rows(RowInputs &in, int64_t row, int64_t n, int q, const float *__restrict__ feat,
+                                          const int32_t *__restrict__ band, const float *__restrict__ target) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int64_t r = row + 8 * h;
+        const bool v = r < n;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            in.x[h][i] = v ? __ldg(reinterpret_cast<const float2 *>(feat + r * kFeat + 8 * i + 2 * q)) : make_float2(0.f, 0.f);
+        in.band[h] = v ? __ldg(band + r) : -1;
+        if (kTrain) in.target[h] = v ? __ldg(target + r) : 0.f;
+    }
+}
+
+// Bound by the latency of its shared-memory loads and products at twelve
+// warps an SM: every fragment of the weights and, in training, of the
+// activations comes from shared memory, four 8x8 matrices per ldmatrix.
+// Activations are stored by row as packed pairs; the weight gradients read
+// them transposed (ldmatrix.trans), so nothing is stored element by element.
+// A tile's inputs are loaded during the weight gradients of the tile before.
+// A training step of 2,752,512 rows: 716 us with 8 warps, activations stored
+// transposed element by element and 32-bit fragment loads; 680 with ldmatrix
+// and two CTAs of 8 warps (128 registers, spilled sums), 622 with one CTA of
+// 12 warps, 541 with the inputs loaded ahead and two column tiles at a time.
+template <bool kTrain>
+__global__ void __launch_bounds__(32 * mlp_warps(kTrain), kTrain ? 1 : 2)
+    k_mlp(int64_t n, int n_tiles, const float *__restrict__ feat, const int32_t *__restrict__ band,
+          const float *__restrict__ target, Weights W, float inv_n, float *__restrict__ score,
+          float *__restrict__ partial) {
+    constexpr int kWarps = mlp_warps(kTrain), kThreads = 32 * kWarps, kTile = mlp_tile(kTrain);
     extern __shared__ __align__(16) unsigned char smem[];
     __nv_bfloat16 *sW1t = reinterpret_cast<__nv_bfloat16 *>(smem);
     __nv_bfloat16 *sW2t = sW1t + kW1Elems;
     __nv_bfloat16 *sW2n = sW2t + kW2Elems;
     float *sb1 = reinterpret_cast<float *>(sW2n + kW2Elems);
     float *sb2 = sb1 + kH, *sw3 = sb2 + kH, *sb3 = sw3 + kH;
-    __nv_bfloat16 *sXT = reinterpret_cast<__nv_bfloat16 *>(sb3 + 4);  // training only
-    __nv_bfloat16 *sH1T = sXT + (size_t)kIn * kLdT;
-    __nv_bfloat16 *sD2T = sH1T + (size_t)kH * kLdT;
-    __nv_bfloat16 *sD1T = sD2T + (size_t)kH * kLdT;
-    float *sRed = reinterpret_cast<float *>(sD1T + (size_t)kH * kLdT);  // [3][kWarps][kH] + [2][kWarps]
+    __nv_bfloat16 *sX = reinterpret_cast<__nv_bfloat16 *>(sb3 + 4);  // training only
+    __nv_bfloat16 *sH1 = sX + (size_t)kTile * kLdX;
+    __nv_bfloat16 *sD2 = sH1 + (size_t)kTile * kLdA;
+    __nv_bfloat16 *sD1 = sD2 + (size_t)kTile * kLdA;
+    float *sRed = reinterpret_cast<float *>(sD1 + (size_t)kTile * kLdA);  // [3][kWarps][kH] + [2][kWarps]
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, q = lane & 3;
+    const int mi = lane >> 3, mr = lane & 7;  // the matrix and row whose address the lane gives an ldmatrix
     {
         const uint4 *s1 = reinterpret_cast<const uint4 *>(W.w1t);
         const uint4 *s2 = reinterpret_cast<const uint4 *>(W.w2t);
@@ -115,7 +180,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp(int64_t n, int n_tiles, con
 
     // training accumulators (per thread, columns 8 nt + 2 q + e)
     float acc_w3[8][2], acc_b2[8][2], acc_b1[8][2];
-    float acc_dw2[4][4], acc_dw1[3][4];
+    float acc_dw[6][4];  // this warp's tiles of dW2 (warps 0 to 7: four) or dW1 (warps 8 to 11: six)
     float acc_b3 = 0.f, acc_loss = 0.f;
     if (kTrain) {
 #pragma unroll
@@ -123,22 +188,17 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp(int64_t n, int n_tiles, con
 #pragma unroll
             for (int e = 0; e < 2; ++e) acc_w3[i][e] = acc_b2[i][e] = acc_b1[i][e] = 0.f;
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < 6; ++i)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) acc_dw2[i][e] = 0.f;
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) acc_dw1[i][e] = 0.f;
+            for (int e = 0; e < 4; ++e) acc_dw[i][e] = 0.f;
     }
 
+    RowInputs in;
+    load_rows<kTrain>(in, (int64_t)blockIdx.x * kTile + warp * 16 + g, n, q, feat, band, target);
     for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
         const int64_t r0 = (int64_t)tile * kTile + warp * 16;
         const int64_t ra = r0 + g, rb = r0 + g + 8;
         const bool va = ra < n, vb = rb < n;
-        int ba = va ? __ldg(band + ra) : -1, bb = vb ? __ldg(band + rb) : -1;
-        if (ba < 0 || ba > 3) ba = -1;  // no band: all-zero one-hot
-        if (bb < 0 || bb > 3) bb = -1;
         const int la = warp * 16 + g, lb = la + 8;  // rows within the CTA tile
 
         // ---- layer 1: z1 = x W1 + b1 -------------------------------------
@@ -148,42 +208,53 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp(int64_t n, int n_tiles, con
 #pragma unroll
             for (int half = 0; half < 2; ++half) {
                 const int c = 16 * kk + 8 * half + 2 * q;
-                const float2 xa = input_pair(feat, ba, va, (int)ra, c);
-                const float2 xb = input_pair(feat, bb, vb, (int)rb, c);
-                const __nv_bfloat16 xa0 = __float2bfloat16_rn(xa.x), xa1 = __float2bfloat16_rn(xa.y);
-                const __nv_bfloat16 xb0 = __float2bfloat16_rn(xb.x), xb1 = __float2bfloat16_rn(xb.y);
-                a1[kk][2 * half] = pack2(xa0, xa1);
-                a1[kk][2 * half + 1] = pack2(xb0, xb1);
-                if (kTrain) {
-                    sXT[c * kLdT + la] = xa0;
-                    sXT[(c + 1) * kLdT + la] = xa1;
-                    sXT[c * kLdT + lb] = xb0;
-                    sXT[(c + 1) * kLdT + lb] = xb1;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    // columns 32 to 35: one-hot band; 36 to 47: zero
+                    const int b = c - kFeat;
+                    const float2 x = kk < 2 ? in.x[h][2 * kk + half]
+                                            : make_float2(b < 4 && b == in.band[h] ? 1.f : 0.f,
+                                                          b < 4 && b + 1 == in.band[h] ? 1.f : 0.f);
+                    a1[kk][2 * half + h] = pack2(__float2bfloat16_rn(x.x), __float2bfloat16_rn(x.y));
+                    if (kTrain) st32(sX + (la + 8 * h) * kLdX + c, a1[kk][2 * half + h]);
                 }
             }
         }
         uint32_t a2[4][4];  // bf16 h1 as layer-2 A fragments
         uint32_t mask1 = 0;
 #pragma unroll
-        for (int nt = 0; nt < 8; ++nt) {
-            const int col = 8 * nt + 2 * q;
-            float d[4] = {sb1[col], sb1[col + 1], sb1[col], sb1[col + 1]};
-            const __nv_bfloat16 *bp = sW1t + (8 * nt + g) * kLdW1 + 2 * q;
+        for (int n0 = 0; n0 < 8; n0 += kChains) {
+            float d[kChains][4];
+            uint32_t b[kChains][4], bx[kChains / 2][4];  // k steps 0 and 1; the third of two column tiles
 #pragma unroll
-            for (int kk = 0; kk < 3; ++kk) mma16816(d, a1[kk], ld32(bp + 16 * kk), ld32(bp + 16 * kk + 8));
-            __nv_bfloat16 h[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                if (d[e] > 0.f) mask1 |= 1u << (4 * nt + e);
-                h[e] = __float2bfloat16_rn(fmaxf(d[e], 0.f));
+            for (int i = 0; i < kChains; ++i) {
+                const float2 bias = *reinterpret_cast<const float2 *>(sb1 + 8 * (n0 + i) + 2 * q);
+                d[i][0] = d[i][2] = bias.x;
+                d[i][1] = d[i][3] = bias.y;
+                ldsm4(b[i], sW1t + (8 * (n0 + i) + mr) * kLdW1 + 8 * mi);
+                if (!(i & 1)) ldsm4(bx[i / 2], sW1t + (8 * (n0 + i + (mi >> 1)) + mr) * kLdW1 + 32 + 8 * (mi & 1));
             }
-            a2[nt >> 1][(nt & 1) * 2] = pack2(h[0], h[1]);
-            a2[nt >> 1][(nt & 1) * 2 + 1] = pack2(h[2], h[3]);
-            if (kTrain) {
-                sH1T[col * kLdT + la] = h[0];
-                sH1T[(col + 1) * kLdT + la] = h[1];
-                sH1T[col * kLdT + lb] = h[2];
-                sH1T[(col + 1) * kLdT + lb] = h[3];
+#pragma unroll
+            for (int i = 0; i < kChains; ++i) mma16816(d[i], a1[0], b[i][0], b[i][1]);
+#pragma unroll
+            for (int i = 0; i < kChains; ++i) mma16816(d[i], a1[1], b[i][2], b[i][3]);
+#pragma unroll
+            for (int i = 0; i < kChains; ++i) mma16816(d[i], a1[2], bx[i / 2][2 * (i & 1)], bx[i / 2][2 * (i & 1) + 1]);
+#pragma unroll
+            for (int i = 0; i < kChains; ++i) {
+                const int nt = n0 + i, col = 8 * nt + 2 * q;
+                __nv_bfloat16 h[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    if (d[i][e] > 0.f) mask1 |= 1u << (4 * nt + e);
+                    h[e] = __float2bfloat16_rn(fmaxf(d[i][e], 0.f));
+                }
+                a2[nt >> 1][(nt & 1) * 2] = pack2(h[0], h[1]);
+                a2[nt >> 1][(nt & 1) * 2 + 1] = pack2(h[2], h[3]);
+                if (kTrain) {
+                    st32(sH1 + la * kLdA + col, a2[nt >> 1][(nt & 1) * 2]);
+                    st32(sH1 + lb * kLdA + col, a2[nt >> 1][(nt & 1) * 2 + 1]);
+                }
             }
         }
         // ---- layer 2: z2 = h1 W2 + b2; output y = relu(z2) w3 + b3 --------
@@ -191,19 +262,27 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp(int64_t n, int n_tiles, con
         uint32_t mask2 = 0;
         float pa = 0.f, pb = 0.f;
 #pragma unroll
-        for (int nt = 0; nt < 8; ++nt) {
-            const int col = 8 * nt + 2 * q;
-            float d[4] = {sb2[col], sb2[col + 1], sb2[col], sb2[col + 1]};
-            const __nv_bfloat16 *bp = sW2t + (8 * nt + g) * kLdW2 + 2 * q;
+        for (int n0 = 0; n0 < 8; n0 += kChains) {
+            float d[kChains][4];
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) mma16816(d, a2[kk], ld32(bp + 16 * kk), ld32(bp + 16 * kk + 8));
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                if (d[e] > 0.f) mask2 |= 1u << (4 * nt + e);
-                h2[nt][e] = fmaxf(d[e], 0.f);
+            for (int i = 0; i < kChains; ++i) {
+                const float2 bias = *reinterpret_cast<const float2 *>(sb2 + 8 * (n0 + i) + 2 * q);
+                d[i][0] = d[i][2] = bias.x;
+                d[i][1] = d[i][3] = bias.y;
             }
-            pa += h2[nt][0] * sw3[col] + h2[nt][1] * sw3[col + 1];
-            pb += h2[nt][2] * sw3[col] + h2[nt][3] * sw3[col + 1];
+            mma_chains(d, a2, sW2t + (8 * n0 + mr) * kLdW2 + 8 * mi);
+#pragma unroll
+            for (int i = 0; i < kChains; ++i) {
+                const int nt = n0 + i;
+                const float2 w3 = *reinterpret_cast<const float2 *>(sw3 + 8 * nt + 2 * q);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    if (d[i][e] > 0.f) mask2 |= 1u << (4 * nt + e);
+                    h2[nt][e] = fmaxf(d[i][e], 0.f);
+                }
+                pa += h2[nt][0] * w3.x + h2[nt][1] * w3.y;
+                pb += h2[nt][2] * w3.x + h2[nt][3] * w3.y;
+            }
         }
         pa += __shfl_xor_sync(0xffffffffu, pa, 1);
         pa += __shfl_xor_sync(0xffffffffu, pa, 2);
@@ -215,11 +294,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp(int64_t n, int n_tiles, con
                 if (va) score[ra] = ya;
                 if (vb) score[rb] = yb;
             }
+            load_rows<kTrain>(in, ra + (int64_t)gridDim.x * kTile, n, q, feat, band, target);
             continue;
         }
         // ---- backward ---------------------------------------------------
-        const float ea = va ? ya - __ldg(target + ra) : 0.f;
-        const float eb = vb ? yb - __ldg(target + rb) : 0.f;
+        const float ea = va ? ya - in.target[0] : 0.f;
+        const float eb = vb ? yb - in.target[1] : 0.f;
         const float dya = 2.f * ea * inv_n, dyb = 2.f * eb * inv_n;
         if (q == 0) {
             acc_loss += ea * ea + eb * eb;
@@ -229,11 +309,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp(int64_t n, int n_tiles, con
 #pragma unroll
         for (int nt = 0; nt < 8; ++nt) {
             const int col = 8 * nt + 2 * q;
+            const float2 w3 = *reinterpret_cast<const float2 *>(sw3 + col);
             float dz[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const float dy = e < 2 ? dya : dyb;
-                dz[e] = (mask2 >> (4 * nt + e)) & 1u ? dy * sw3[col + (e & 1)] : 0.f;
+                dz[e] = (mask2 >> (4 * nt + e)) & 1u ? dy * (e & 1 ? w3.y : w3.x) : 0.f;
             }
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
@@ -245,86 +326,85 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp(int64_t n, int n_tiles, con
             for (int e = 0; e < 4; ++e) hb[e] = __float2bfloat16_rn(dz[e]);
             ad[nt >> 1][(nt & 1) * 2] = pack2(hb[0], hb[1]);
             ad[nt >> 1][(nt & 1) * 2 + 1] = pack2(hb[2], hb[3]);
-            sD2T[col * kLdT + la] = hb[0];
-            sD2T[(col + 1) * kLdT + la] = hb[1];
-            sD2T[col * kLdT + lb] = hb[2];
-            sD2T[(col + 1) * kLdT + lb] = hb[3];
+            st32(sD2 + la * kLdA + col, ad[nt >> 1][(nt & 1) * 2]);
+            st32(sD2 + lb * kLdA + col, ad[nt >> 1][(nt & 1) * 2 + 1]);
         }
         // dh1 = dz2 W2^T, dz1 = dh1 * [z1 > 0]
 #pragma unroll
-        for (int nt = 0; nt < 8; ++nt) {
-            const int col = 8 * nt + 2 * q;
-            float d[4] = {0.f, 0.f, 0.f, 0.f};
-            const __nv_bfloat16 *bp = sW2n + (8 * nt + g) * kLdW2 + 2 * q;
+        for (int n0 = 0; n0 < 8; n0 += kChains) {
+            float d[kChains][4];
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) mma16816(d, ad[kk], ld32(bp + 16 * kk), ld32(bp + 16 * kk + 8));
-            __nv_bfloat16 hb[4];
+            for (int i = 0; i < kChains; ++i) d[i][0] = d[i][1] = d[i][2] = d[i][3] = 0.f;
+            mma_chains(d, ad, sW2n + (8 * n0 + mr) * kLdW2 + 8 * mi);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const float dz = (mask1 >> (4 * nt + e)) & 1u ? d[e] : 0.f;
-                if (e < 2) acc_b1[nt][e] += dz; else acc_b1[nt][e - 2] += dz;
-                hb[e] = __float2bfloat16_rn(dz);
+            for (int i = 0; i < kChains; ++i) {
+                const int nt = n0 + i, col = 8 * nt + 2 * q;
+                __nv_bfloat16 hb[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float dz = (mask1 >> (4 * nt + e)) & 1u ? d[i][e] : 0.f;
+                    acc_b1[nt][e & 1] += dz;
+                    hb[e] = __float2bfloat16_rn(dz);
+                }
+                st32(sD1 + la * kLdA + col, pack2(hb[0], hb[1]));
+                st32(sD1 + lb * kLdA + col, pack2(hb[2], hb[3]));
             }
-            sD1T[col * kLdT + la] = hb[0];
-            sD1T[(col + 1) * kLdT + la] = hb[1];
-            sD1T[col * kLdT + lb] = hb[2];
-            sD1T[(col + 1) * kLdT + lb] = hb[3];
         }
+        // the next tile's inputs arrive during the weight gradients
+        load_rows<kTrain>(in, ra + (int64_t)gridDim.x * kTile, n, q, feat, band, target);
         __syncthreads();
-        // ---- weight gradients over the tile's 128 rows ------------------
-        // dW2[m][n] = sum_r h1[r][m] dz2[r][n]: warp -> m tile warp/2, n tiles 4 (warp%2) + i
-        {
-            const int mt = warp >> 1;
-#pragma unroll
+        // ---- weight gradients over the tile's rows ----------------------
+        // Fragments from the row-major tiles, transposed: A (features m, rows
+        // k) matrix i at rows 8 (i / 2), features 8 (i % 2); B (rows k,
+        // features n of two tiles) matrix i at rows 8 (i % 2), features 8 (i / 2)
+        if (warp < 8) {
+            // dW2[m][n] = sum_r h1[r][m] dz2[r][n]: m tile warp/2, n tiles 4 (warp%2) + i
+            const __nv_bfloat16 *ah = sH1 + (8 * (mi >> 1) + mr) * kLdA + 16 * (warp >> 1) + 8 * (mi & 1);
+            const __nv_bfloat16 *bd = sD2 + (8 * (mi & 1) + mr) * kLdA + 32 * (warp & 1) + 8 * (mi >> 1);
+#pragma unroll 4
             for (int ks = 0; ks < kTile / 16; ++ks) {
-                const __nv_bfloat16 *ap = sH1T + (16 * mt + g) * kLdT + 16 * ks + 2 * q;
-                const uint32_t a[4] = {ld32(ap), ld32(ap + 8 * kLdT), ld32(ap + 8), ld32(ap + 8 * kLdT + 8)};
+                uint32_t a[4], b[4];
+                ldsm4t(a, ah + 16 * ks * kLdA);
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int nt = 4 * (warp & 1) + i;
-                    const __nv_bfloat16 *bp = sD2T + (8 * nt + g) * kLdT + 16 * ks + 2 * q;
-                    mma16816(acc_dw2[i], a, ld32(bp), ld32(bp + 8));
+                for (int i = 0; i < 4; i += 2) {
+                    ldsm4t(b, bd + 16 * ks * kLdA + 8 * i);
+                    mma16816(acc_dw[i], a, b[0], b[1]);
+                    mma16816(acc_dw[i + 1], a, b[2], b[3]);
+                }
+            }
+        } else {
+            // dW1[m][n] = sum_r x[r][m] dz1[r][n]: n tiles 2 (warp - 8) + i, m tiles 0 to 2
+            const __nv_bfloat16 *ax = sX + (8 * (mi >> 1) + mr) * kLdX + 8 * (mi & 1);
+            const __nv_bfloat16 *bz = sD1 + (8 * (mi & 1) + mr) * kLdA + 16 * (warp - 8) + 8 * (mi >> 1);
+#pragma unroll 4
+            for (int ks = 0; ks < kTile / 16; ++ks) {
+                uint32_t a[4], b[4];
+                ldsm4t(b, bz + 16 * ks * kLdA);
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    ldsm4t(a, ax + 16 * ks * kLdX + 16 * i);
+                    mma16816(acc_dw[2 * i], a, b[0], b[1]);
+                    mma16816(acc_dw[2 * i + 1], a, b[2], b[3]);
                 }
             }
         }
-        // dW1[m][n] = sum_r x[r][m] dz1[r][n]: 3 m tiles x 8 n tiles, 3 per warp
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            const int id = 3 * warp + i, mt = id >> 3, nt = id & 7;
-#pragma unroll
-            for (int ks = 0; ks < kTile / 16; ++ks) {
-                const __nv_bfloat16 *ap = sXT + (16 * mt + g) * kLdT + 16 * ks + 2 * q;
-                const uint32_t a[4] = {ld32(ap), ld32(ap + 8 * kLdT), ld32(ap + 8), ld32(ap + 8 * kLdT + 8)};
-                const __nv_bfloat16 *bp = sD1T + (8 * nt + g) * kLdT + 16 * ks + 2 * q;
-                mma16816(acc_dw1[i], a, ld32(bp), ld32(bp + 8));
-            }
-        }
-        __syncthreads();  // the transposed tiles are rewritten by the next tile
+        __syncthreads();  // the activations are rewritten by the next tile
     }
     if (!kTrain) return;
 
     // ---- per-CTA partial gradient, written in a fixed order --------------
     float *out = partial + (size_t)blockIdx.x * (kP + 1);
-    {
-        const int mt = warp >> 1;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int nt = 4 * (warp & 1) + i;
-            const int m = 16 * mt + g, c = 8 * nt + 2 * q;
-            out[oW2 + m * kH + c] = acc_dw2[i][0];
-            out[oW2 + m * kH + c + 1] = acc_dw2[i][1];
-            out[oW2 + (m + 8) * kH + c] = acc_dw2[i][2];
-            out[oW2 + (m + 8) * kH + c + 1] = acc_dw2[i][3];
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        const int id = 3 * warp + i, mt = id >> 3, nt = id & 7;
-        const int m = 16 * mt + g, c = 8 * nt + 2 * q;
-        out[oW1 + m * kH + c] = acc_dw1[i][0];
-        out[oW1 + m * kH + c + 1] = acc_dw1[i][1];
-        out[oW1 + (m + 8) * kH + c] = acc_dw1[i][2];
-        out[oW1 + (m + 8) * kH + c + 1] = acc_dw1[i][3];
+    for (int i = 0; i < 6; ++i) {
+        // tile i: rows m and m + 8, columns c and c + 1 of W2 or W1
+        if (warp < 8 && i >= 4) break;
+        const int o = warp < 8 ? oW2 : oW1;
+        const int m = 16 * (warp < 8 ? warp >> 1 : i >> 1) + g;
+        const int c = 8 * (warp < 8 ? 4 * (warp & 1) + i : 2 * (warp - 8) + (i & 1)) + 2 * q;
+        out[o + m * kH + c] = acc_dw[i][0];
+        out[o + m * kH + c + 1] = acc_dw[i][1];
+        out[o + (m + 8) * kH + c] = acc_dw[i][2];
+        out[o + (m + 8) * kH + c + 1] = acc_dw[i][3];
     }
     // column sums: over the 8 lanes of equal q, then over warps via shared memory
     float *rw3 = sRed, *rb2 = rw3 + kWarps * kH, *rb1 = rb2 + kWarps * kH, *rs = rb1 + kWarps * kH;
@@ -472,9 +552,9 @@ int mfail(cs_mlp *m, int code, const char *fmt, ...) {
 
 bool aligned(const void *p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; }
 
-int grid_for(const cs_mlp *m, int64_t n) {
-    const int64_t tiles = (n + kTile - 1) / kTile;
-    return (int)std::min<int64_t>(tiles, 2LL * m->n_sm);
+int grid_for(const cs_mlp *m, int64_t n, bool train) {
+    const int64_t tiles = (n + mlp_tile(train) - 1) / mlp_tile(train);
+    return (int)std::min<int64_t>(tiles, (train ? 1LL : 2LL) * m->n_sm);
 }
 
 int refresh_copies(cs_mlp *m) {
@@ -581,9 +661,9 @@ int cs_mlp_forward(cs_mlp *m, int64_t n, const float *feat, const int32_t *band,
     if (!feat || !band || !score_out || !aligned(feat, 8) || !aligned(band, 4) || !aligned(score_out, 4))
         return mfail(m, CS_ERR_ARG, "NULL or misaligned array");
     MLP_CUDA(m, cudaSetDevice(m->device));
-    const int tiles = (int)((n + kTile - 1) / kTile);
+    const int tiles = (int)((n + mlp_tile(false) - 1) / mlp_tile(false));
     Weights W{m->w1t, m->w2t, m->w2n, m->master};
-    k_mlp<false><<<grid_for(m, n), kThreads, kSmemWeights, m->stream>>>(n, tiles, feat, band, nullptr, W, 0.f,
+    k_mlp<false><<<grid_for(m, n, false), 32 * mlp_warps(false), kSmemWeights, m->stream>>>(n, tiles, feat, band, nullptr, W, 0.f,
                                                                        score_out, nullptr);
     MLP_CUDA(m, cudaGetLastError());
     return CS_OK;
@@ -598,7 +678,7 @@ int cs_mlp_train_step(cs_mlp *m, int64_t n, const float *feat, const int32_t *ba
     if (!feat || !band || !target || !aligned(feat, 8) || !aligned(band, 4) || !aligned(target, 4))
         return mfail(m, CS_ERR_ARG, "NULL or misaligned array");
     MLP_CUDA(m, cudaSetDevice(m->device));
-    const int grid = grid_for(m, n);
+    const int grid = grid_for(m, n, true);
     if (grid > m->n_part_cap) {
         MLP_CUDA(m, cudaStreamSynchronize(m->stream));
         cudaFree(m->partial);
@@ -607,9 +687,9 @@ int cs_mlp_train_step(cs_mlp *m, int64_t n, const float *feat, const int32_t *ba
         MLP_CUDA(m, cudaMalloc(&m->partial, (size_t)grid * (kP + 1) * 4));
         m->n_part_cap = grid;
     }
-    const int tiles = (int)((n + kTile - 1) / kTile);
+    const int tiles = (int)((n + mlp_tile(true) - 1) / mlp_tile(true));
     Weights W{m->w1t, m->w2t, m->w2n, m->master};
-    k_mlp<true><<<grid, kThreads, kSmemTrain, m->stream>>>(n, tiles, feat, band, target, W, (float)(1.0 / (double)n),
+    k_mlp<true><<<grid, 32 * mlp_warps(true), kSmemTrain, m->stream>>>(n, tiles, feat, band, target, W, (float)(1.0 / (double)n),
                                                           nullptr, m->partial);
     MLP_CUDA(m, cudaGetLastError());
     const int64_t t = m->steps + 1;
