@@ -12,10 +12,17 @@
 //      1080p as 7 + 6) leaves every tile's pairs in (depth, splat id) order.
 // Each radix pass is reduce-then-scan (histogram of each digit per block,
 // one CTA per digit scanning its row of block counts, scatter): no
-// inter-block waits, and the order is deterministic.
+// inter-block waits, and the order is deterministic.  Sorts of up to eight
+// blocks run in one launch of a thread-block cluster.
+#include <cooperative_groups.h>
+
+#include <algorithm>
+
 #include "cs_internal.cuh"
 
 namespace cs {
+
+namespace cg = cooperative_groups;
 
 // ---------------------------------------------------------------------------
 // exclusive scan of uint32 (three kernels: tile sums, spine, down-sweep)
@@ -321,6 +328,166 @@ __global__ void __launch_bounds__(kRadixThreads, 3) k_radix_scatter(
     }
 }
 
+// The whole sort of up to kClusterBlocks blocks in one launch: a cluster of
+// CTAs, one per 4,096 elements, runs every pass, reading the other CTAs'
+// digit counts from their shared memory and handing the elements on through
+// global memory (L2), with two cluster barriers a pass.  Such sorts are
+// bound by launches: three kernels a pass, each shorter than the gap to the
+// next.  Same digits, same order.  A 256x256 frame of 16,384 splats: 194 ->
+// 162 us; a training frame of 12,291 splats: 424 -> 394 us.
+constexpr int kClusterBlocks = 8;  // the portable cluster size
+
+// Digit width of pass p of `passes` over `bits` bits, from bit `shift` on.
+__host__ __device__ inline int radix_width(int bits, int shift, int passes, int p) {
+    const int w = (bits - shift + (passes - p) - 1) / (passes - p);
+    return w < 4 ? 4 : w;
+}
+
+template <typename K>
+__global__ void __launch_bounds__(kRadixThreads) k_radix_cluster(K *k0, uint32_t *v0, K *k1, uint32_t *v1, uint32_t n,
+                                                                 int bits, int passes, bool iota,
+                                                                 const uint32_t *__restrict__ gsrc,
+                                                                 uint32_t *__restrict__ gdst) {
+    __shared__ uint32_t wcnt[kRadixWarps][kRadixDigits];  // running counts, then warp offsets
+    __shared__ uint32_t dcnt[kRadixDigits];               // this block's digit counts, read by the cluster
+    __shared__ uint32_t dstart[kRadixDigits], gbase[kRadixDigits];
+    __shared__ uint32_t total;
+    extern __shared__ __align__(16) unsigned char cluster_dyn[];
+    uint32_t *sval = reinterpret_cast<uint32_t *>(cluster_dyn);
+    K *skey = reinterpret_cast<K *>(cluster_dyn + kRadixTile * sizeof(uint32_t));
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank(), blocks = (int)cluster.num_blocks();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t lt = (1u << lane) - 1u;
+    const uint32_t blk0 = (uint32_t)rank * kRadixTile, base = blk0 + warp * kRadixWarpTile;
+    constexpr int kPer = kRadixDigits / kRadixThreads;  // digits per thread
+    for (int p = 0, shift = 0; p < passes; ++p) {
+        const int width = radix_width(bits, shift, passes, p);
+        const uint32_t mask = (1u << width) - 1u;
+        const K *ki = p & 1 ? k1 : k0;
+        const uint32_t *vi = p & 1 ? v1 : v0;
+        K *ko = p & 1 ? k0 : k1;
+        uint32_t *vo = p & 1 ? v0 : v1;
+        for (int d = threadIdx.x; d < kRadixWarps * kRadixDigits; d += kRadixThreads) (&wcnt[0][0])[d] = 0;
+        K k[kRadixItems];
+        uint32_t v[kRadixItems], dr[kRadixItems];
+#pragma unroll
+        for (int r = 0; r < kRadixItems; ++r) {
+            // past L1: another CTA of the cluster wrote them in the pass before
+            const uint32_t i = base + r * 32 + lane;
+            k[r] = i < n ? __ldcg(ki + i) : (K)0;
+            v[r] = i >= n ? 0u : (p == 0 && iota ? i : __ldcg(vi + i));
+        }
+        __syncthreads();
+        // stable rank within the warp's 512 elements, as k_radix_scatter
+#pragma unroll
+        for (int r = 0; r < kRadixItems; ++r) {
+            const bool ok = base + r * 32 + lane < n;
+            const uint32_t d = ok ? (uint32_t)(k[r] >> shift) & mask : (uint32_t)kRadixDigits;
+            unsigned peers = __ballot_sync(0xffffffffu, ok);
+            for (int b = 0; b < width; ++b) {
+                const unsigned m = __ballot_sync(0xffffffffu, (d >> b) & 1u);
+                peers &= ((d >> b) & 1u) ? m : ~m;
+            }
+            const uint32_t before = ok ? wcnt[warp][d] : 0u;
+            __syncwarp();
+            if (ok && (peers & lt) == 0u) wcnt[warp][d] = before + __popc(peers);
+            __syncwarp();
+            dr[r] = d | ((before + __popc(peers & lt)) << 16);
+        }
+        __syncthreads();
+        uint32_t mine[kPer], tot = 0;
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const int d = threadIdx.x * kPer + j;
+            uint32_t run = 0;
+#pragma unroll
+            for (int w = 0; w < kRadixWarps; ++w) {
+                const uint32_t c = wcnt[w][d];
+                wcnt[w][d] = run;
+                run += c;
+            }
+            dcnt[d] = mine[j] = run;
+            tot += run;
+        }
+        cluster.sync();  // every block's digit counts are there
+        uint32_t pre[kPer], all[kPer], gtot = 0;
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) pre[j] = all[j] = 0;
+        for (int b = 0; b < blocks; ++b) {
+            const uint32_t *other = cluster.map_shared_rank(dcnt, b);
+#pragma unroll
+            for (int j = 0; j < kPer; ++j) {
+                const uint32_t c = other[threadIdx.x * kPer + j];
+                if (b < rank) pre[j] += c;
+                all[j] += c;
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) gtot += all[j];
+        uint32_t ex = block_excl_scan(tot, &total), gex = block_excl_scan(gtot, &total);
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const int d = threadIdx.x * kPer + j;
+            dstart[d] = ex;
+            gbase[d] = gex + pre[j];
+            ex += mine[j];
+            gex += all[j];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < kRadixItems; ++r) {
+            const uint32_t d = dr[r] & 0xFFFFu;
+            if (d < (uint32_t)kRadixDigits) {
+                const uint32_t lp = dstart[d] + wcnt[warp][d] + (dr[r] >> 16);
+                skey[lp] = k[r];
+                sval[lp] = v[r];
+            }
+        }
+        __syncthreads();
+        const uint32_t cnt = n > blk0 ? min((uint32_t)kRadixTile, n - blk0) : 0u;
+        const bool last = p == passes - 1;
+        for (uint32_t q = threadIdx.x; q < cnt; q += kRadixThreads) {
+            const K key = skey[q];
+            const uint32_t d = (uint32_t)(key >> shift) & mask;
+            const uint32_t g = gbase[d] + (q - dstart[d]);
+            const uint32_t val = sval[q];
+            if (!in_bounds(g < n, kChkSort)) continue;
+            ko[g] = key;
+            vo[g] = val;
+            if (last && gdst && in_bounds(val < n, kChkSort)) gdst[g] = gsrc[val];
+        }
+        shift += width;
+        cluster.sync();  // the pass is written, and nobody reads these counts any more
+    }
+}
+
+template <typename K>
+static int radix_cluster(K *k0, uint32_t *v0, K *k1, uint32_t *v1, uint32_t n, uint32_t nb, int bits, int passes,
+                         bool iota, const uint32_t *gsrc, uint32_t *gdst, cudaStream_t st) {
+    constexpr int kDyn = kRadixTile * (int)(sizeof(uint32_t) + sizeof(K));
+    static int configured_device = -1;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (configured_device != dev) {
+        cudaFuncSetAttribute(k_radix_cluster<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDyn);
+        configured_device = dev;
+    }
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = nb;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = nb;
+    cfg.blockDim = kRadixThreads;
+    cfg.dynamicSmemBytes = kDyn;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k_radix_cluster<K>, k0, v0, k1, v1, n, bits, passes, iota, gsrc, gdst);
+    return 1;
+}
+
 size_t radix_scratch_words(size_t n) {
     size_t nb = (n + kRadixTile - 1) / kRadixTile;
     if (nb == 0) nb = 1;
@@ -361,14 +528,17 @@ static int radix_sort(K *k0, uint32_t *v0, K *k1, uint32_t *v1, uint32_t n, int 
     const uint32_t nb = (n + kRadixTile - 1) / kRadixTile;
     // fewest passes of at most 9 bits, near-equal widths (4 bits at least)
     const int passes = (bits + kRadixMaxBits - 1) / kRadixMaxBits;
+    if (nb <= (uint32_t)kClusterBlocks) {
+        *in_second = passes & 1;
+        return radix_cluster<K>(k0, v0, k1, v1, n, nb, bits, passes, iota_values, gsrc, gdst, st);
+    }
     int cur = 0;
     for (int p = 0, shift = 0; p < passes; ++p) {
         const K *ki = cur ? k1 : k0;
         const uint32_t *vi = p == 0 && iota_values ? nullptr : (cur ? v1 : v0);
         K *ko = cur ? k0 : k1;
         uint32_t *vo = cur ? v0 : v1;
-        const int left = bits - shift;
-        const int width = std::max(4, (left + (passes - p) - 1) / (passes - p));
+        const int width = radix_width(bits, shift, passes, p);
         const bool last = p == passes - 1;
         const uint32_t *gs = last ? gsrc : nullptr;
         uint32_t *gd = last ? gdst : nullptr;
