@@ -62,14 +62,21 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_spine(uint32_t *__restric
                                                              uint32_t seq) {
     __shared__ uint32_t total;
     uint32_t carry = 0;
-    for (uint32_t base = 0; base < nb; base += kScanThreads) {
-        uint32_t i = base + threadIdx.x;
-        uint32_t v = i < nb ? sums[i] : 0u;
-        uint32_t ex = block_excl_scan(v, &total);
-        if (i < nb) sums[i] = carry + ex;
-        __syncthreads();
+    for (uint32_t base = 0; base < nb; base += kScanTile) {
+        const uint32_t i0 = base + threadIdx.x * kScanItems;
+        uint32_t v[kScanItems], sum = 0;
+#pragma unroll
+        for (int k = 0; k < kScanItems; ++k) {
+            v[k] = i0 + k < nb ? sums[i0 + k] : 0u;
+            sum += v[k];
+        }
+        uint32_t ex = block_excl_scan(sum, &total) + carry;
+#pragma unroll
+        for (int k = 0; k < kScanItems; ++k) {
+            if (i0 + k < nb) sums[i0 + k] = ex;
+            ex += v[k];
+        }
         carry += total;
-        __syncthreads();
     }
     if (threadIdx.x == 0) {
         sums[nb] = carry;
@@ -627,79 +634,159 @@ __global__ void __launch_bounds__(256) k_emit_pairs(uint32_t n, const uint32_t *
     emit_splat_pairs(bins[i], s, pair_off[i], pair_off[i + 1], rec, tiles_x, ptile, pval, n_tiles, pair_off[n]);
 }
 
-// Pair emission fused with the down-sweep of the pair-count scan: block b
-// takes the kScanTile splats from b kScanTile in depth order, in kScanItems
-// rounds of kScanThreads consecutive splats (one per thread, coalesced); its
-// offset comes from the scanned block sums, each round is scanned in the
-// block, so no per-splat offset array is written or read.  A splat whose
-// tiles fit a 3x3 window (at most nine pairs) is written by its thread; a
-// larger one is queued in shared memory and written by a whole warp, lane l
-// taking its tiles l, l + 32, ... in row-major order (coalesced stores, no
-// warp waiting on one lane's long loop): exactly the pairs emit_splat_pairs
-// writes.
-__global__ void __launch_bounds__(kScanThreads) k_emit_pairs_scan(uint32_t n, const uint32_t *__restrict__ order,
-                                                                 const uint32_t *__restrict__ bins,
-                                                                 const uint32_t *__restrict__ sums,
-                                                                 const float4 *__restrict__ rec, int tiles_x,
-                                                                 uint32_t n_tiles, uint16_t *__restrict__ ptile,
-                                                                 uint32_t *__restrict__ pval,
-                                                                 uint2 *__restrict__ ranges,
-                                                                 int32_t *__restrict__ blend_meta) {
-    __shared__ uint32_t total, n_large;
-    for (uint32_t k = blockIdx.x * kScanThreads + threadIdx.x; k < n_tiles; k += gridDim.x * kScanThreads)
-        ranges[k] = make_uint2(0u, 0u);
-    if (blockIdx.x == 0 && threadIdx.x < kBlendMetaWords) blend_meta[threadIdx.x] = 0;
-    const uint32_t n_pairs = CS_CHECKS ? sums[gridDim.x] : 0xFFFFFFFFu;  // the scan's total
-    __shared__ uint4 s_large[kScanThreads];  // splat id, first pair, tile x0 | y0 << 16, tiles per row
-    __shared__ uint32_t s_cnt[kScanThreads];  // its pairs
-    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    uint32_t carry = sums[blockIdx.x];
-    if (t == 0) n_large = 0u;
-#pragma unroll 1
-    for (int r = 0; r < kScanItems; ++r) {
-        const uint32_t i = blockIdx.x * kScanTile + r * kScanThreads + t;
-        const uint32_t b = i < n ? bins[i] : 0u;
-        const uint32_t c = bin_count(b);
-        const uint32_t o = carry + block_excl_scan(c, &total);
-        if (c && in_bounds(order[i] < n, kChkSplat)) {
-            const uint32_t s = order[i];
-            if (!(b & kBinLarge)) {
-                emit_splat_pairs(b, s, o, o + c, rec, tiles_x, ptile, pval, n_tiles, n_pairs);
-            } else {
-                const float4 r3 = rec[(size_t)s * kRecVec];  // reach x, reach y, log2 o, C
-                const uint32_t rx = __float_as_uint(r3.x), ry = __float_as_uint(r3.y);
-                const uint32_t tx0 = (rx & 0xFFFFu) >> 4, ty0 = (ry & 0xFFFFu) >> 4;
-                const uint32_t q = atomicAdd(&n_large, 1u);  // queue order: any (own output range)
-                s_large[q] = make_uint4(s, o, tx0 | (ty0 << 16), ((rx >> 16) >> 4) - tx0 + 1u);
-                s_cnt[q] = c;
-            }
+// Pair emission fused with the down-sweep of the pair-count scan.  A block
+// takes 256 kRounds splats in depth order, warp w the 32 kRounds from
+// w 32 kRounds on; the warp's offset is the scanned block sum plus the
+// totals of the warps before it, so there is one barrier and no per-splat
+// offset array.  Each round of 32 splats is scanned in the warp and its
+// pairs are written 32 at a time, one per lane: the lanes whose splats have
+// pairs leave them compacted in shared memory, a bit per splat start in the
+// window of 32 pairs (one reduction) tells each lane its splat, and the pair's rank among the
+// splat's tiles its tile (row-major; a 3x3 mask by a table of the positions
+// of its set bits).  Exactly the pairs emit_splat_pairs writes, in their
+// order.
+// Bound by instruction issue (about 150 per 32 splats and their pairs).
+// 42.5 M pairs of 22.7 M splats: 228 -> 178 us against 1,024-thread blocks
+// with three barriers a round, small splats written by their own threads and
+// larger ones queued; the sums before it 27 -> 18 us (16-byte loads).
+constexpr int kEmitThreads = 256;
+constexpr int kEmitWarps = kEmitThreads / 32;
+// Blocks of 4,096 splats leave SMs idle below a few million splats (202,738
+// splats are 50 blocks: 21 us, 13 with blocks of 1,024); above, the smaller
+// blocks would only lengthen the one-block scan of the sums.
+constexpr int kEmitRounds = 16, kEmitFewRounds = 4;
+constexpr size_t kEmitFewSplats = (size_t)1 << 22;
+
+template <int kRounds>
+__global__ void __launch_bounds__(kEmitThreads) k_bin_sums(const uint32_t *__restrict__ bins, uint32_t n,
+                                                           uint32_t *__restrict__ sums) {
+    __shared__ uint32_t wsum[kEmitWarps];
+    const uint32_t base = blockIdx.x * (kEmitThreads * kRounds);
+    uint32_t v = 0;
+#pragma unroll
+    for (int j = 0; j < kRounds / 4; ++j) {
+        const uint32_t i = base + (j * kEmitThreads + threadIdx.x) * 4u;
+        if (i + 4u <= n) {
+            const uint4 w = __ldg(reinterpret_cast<const uint4 *>(bins + i));  // (the words start 16-byte aligned)
+            v += bin_count(w.x) + bin_count(w.y) + bin_count(w.z) + bin_count(w.w);
+        } else {
+            for (uint32_t k = i; k < n; ++k) v += bin_count(bins[k]);
         }
-        carry += total;
-        __syncthreads();
-        const uint32_t nl = n_large;
-        for (uint32_t q = warp; q < nl; q += kScanThreads / 32) {
-            const uint4 L = s_large[q];  // splat id, first pair, tile x0 | y0 << 16, tiles per row
-            const uint32_t cnt = s_cnt[q];
-            if (!in_bounds(L.y + cnt <= n_pairs, kChkPair)) continue;
-            for (uint32_t k = lane; k < cnt; k += 32) {
-                const uint32_t row = k / L.w, col = k - row * L.w;
-                const uint32_t tile = ((L.z >> 16) + row) * (uint32_t)tiles_x + (L.z & 0xFFFFu) + col;
-                if (!in_bounds(tile < n_tiles, kChkTile)) continue;
-                ptile[L.y + k] = (uint16_t)tile;
-                pval[L.y + k] = L.x;
-            }
-        }
-        __syncthreads();  // the queue is refilled by the next round
-        if (t == 0) n_large = 0u;
+    }
+    v = __reduce_add_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint32_t t = 0;
+        for (int w = 0; w < kEmitWarps; ++w) t += wsum[w];
+        sums[blockIdx.x] = t;
     }
 }
 
-size_t bin_scan_blocks(size_t n) { return (n + kScanTile - 1) / kScanTile; }
+template <int kRounds>
+__global__ void __launch_bounds__(kEmitThreads, 8)
+    k_emit_pairs_scan(uint32_t n, const uint32_t *__restrict__ order, const uint32_t *__restrict__ bins,
+                      const uint32_t *__restrict__ sums, const float4 *__restrict__ rec, int tiles_x,
+                      uint32_t n_tiles, uint16_t *__restrict__ ptile, uint32_t *__restrict__ pval,
+                      uint2 *__restrict__ ranges, int32_t *__restrict__ blend_meta) {
+    __shared__ uint4 stage[kEmitWarps][32];  // splat id, first pair, tile x0 | y0 << 16, mask or large | tiles per row
+    __shared__ uint32_t nth[512];            // positions of a mask's first eight set bits, four bits each
+    __shared__ uint32_t wsum[kEmitWarps];
+    for (uint32_t k = blockIdx.x * kEmitThreads + threadIdx.x; k < n_tiles; k += gridDim.x * kEmitThreads)
+        ranges[k] = make_uint2(0u, 0u);
+    if (blockIdx.x == 0 && threadIdx.x < kBlendMetaWords) blend_meta[threadIdx.x] = 0;
+    const uint32_t n_pairs = CS_CHECKS ? sums[gridDim.x] : 0xFFFFFFFFu;  // the scan's total
+    for (uint32_t m = threadIdx.x; m < 512u; m += kEmitThreads) {
+        uint32_t x = 0, k = 0;
+        for (uint32_t j = 0; j < 9u; ++j)
+            if ((m >> j) & 1u) {
+                if (k < 8u) x |= j << (4u * k);
+                ++k;
+            }
+        nth[m] = x;
+    }
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t lt = (1u << lane) - 1u;
+    const uint32_t base = (blockIdx.x * kEmitWarps + warp) * (32u * kRounds);
+    uint32_t mine = 0;
+#pragma unroll
+    for (int r = 0; r < kRounds; ++r) mine += base + r * 32 + lane < n ? bin_count(bins[base + r * 32 + lane]) : 0u;
+    mine = __reduce_add_sync(0xffffffffu, mine);
+    if (lane == 0) wsum[warp] = mine;
+    __syncthreads();
+    if (mine == 0u) return;
+    uint32_t o0 = sums[blockIdx.x];
+    for (int w = 0; w < warp; ++w) o0 += wsum[w];
+    // bin words are read two rounds ahead, splat ids one
+    uint32_t i = base + lane;
+    uint32_t b = i < n ? bins[i] : 0u, b1 = i + 32u < n ? bins[i + 32] : 0u;
+    uint32_t s = bin_count(b) ? order[i] : 0u;
+#pragma unroll 1
+    for (int r = 0; r < kRounds; ++r, i += 32) {
+        const uint32_t b2 = r + 2 < kRounds && i + 64u < n ? bins[i + 64] : 0u;
+        const uint32_t s1 = r + 1 < kRounds && bin_count(b1) ? order[i + 32] : 0u;
+        const uint32_t c = bin_count(b);
+        const uint32_t incl = warp_inclusive_scan(c), first = incl - c;
+        const uint32_t pairs = __shfl_sync(0xffffffffu, incl, 31);
+        const unsigned have = __ballot_sync(0xffffffffu, c != 0u);
+        if (c) {
+            uint4 e = make_uint4(s, first, (b & 0xFFu) | ((b & 0xFF00u) << 8), (b >> 16) & 0x1FFu);
+            if ((b & kBinLarge) && in_bounds(s < n, kChkSplat)) {
+                const float4 q = rec[(size_t)s * kRecVec];  // reach x, reach y, log2 o, C
+                const uint32_t rx = __float_as_uint(q.x), ry = __float_as_uint(q.y);
+                const uint32_t x0 = (rx & 0xFFFFu) >> 4, y0 = (ry & 0xFFFFu) >> 4;
+                e.z = x0 | (y0 << 16);
+                e.w = kBinLarge | (((rx >> 16) >> 4) - x0 + 1u);
+            }
+            stage[warp][__popc(have & lt)] = e;
+        }
+        __syncwarp();
+        uint32_t started = 0;
+        for (uint32_t w0 = 0; w0 < pairs; w0 += 32u) {
+            const unsigned starts = __reduce_or_sync(0xffffffffu, c && first - w0 < 32u ? 1u << (first - w0) : 0u);
+            const uint32_t p = w0 + lane;
+            const uint32_t owner = started + __popc(starts & (lt | (1u << lane))) - 1u;
+            started += __popc(starts);
+            if (p >= pairs) continue;
+            const uint4 e = stage[warp][owner];
+            const uint32_t k = p - e.y;  // rank among the splat's tiles
+            uint32_t row, col;
+            if (e.w & kBinLarge) {
+                // k / width: exact for k < 2^16 (the quotient is at least half
+                // a width's inverse away from an integer)
+                const uint32_t width = e.w & ~kBinLarge;
+                row = (uint32_t)(((float)k + 0.5f) * (1.0f / (float)width));
+                col = k - row * width;
+            } else {
+                const uint32_t at = k < 8u ? (nth[e.w] >> (4u * k)) & 15u : 8u;
+                row = at / 3u;
+                col = at - 3u * row;
+            }
+            const uint32_t tile = ((e.z >> 16) + row) * (uint32_t)tiles_x + (e.z & 0xFFFFu) + col;
+            const uint32_t o = o0 + p;
+            if (in_bounds(o < n_pairs, kChkPair) && in_bounds(e.x < n, kChkSplat) && in_bounds(tile < n_tiles, kChkTile)) {
+                ptile[o] = (uint16_t)tile;
+                pval[o] = e.x;
+            }
+        }
+        __syncwarp();  // the staged splats are replaced by the next round's
+        o0 += pairs;
+        b = b1;
+        b1 = b2;
+        s = s1;
+    }
+}
+
+// splats of a block of the two kernels above
+static uint32_t emit_tile(size_t n) { return kEmitThreads * (n <= kEmitFewSplats ? kEmitFewRounds : kEmitRounds); }
+
+size_t bin_scan_blocks(size_t n) { return (n + emit_tile(n) - 1) / emit_tile(n); }
 
 int bin_scan_sums(const uint32_t *bins, uint32_t n, uint32_t *sums, uint32_t *host, uint32_t seq, cudaStream_t st) {
     if (n == 0) return 0;
     const uint32_t nb = (uint32_t)bin_scan_blocks(n);
-    k_scan_reduce<1><<<nb, kScanThreads, 0, st>>>(bins, n, sums);
+    if (n <= kEmitFewSplats) k_bin_sums<kEmitFewRounds><<<nb, kEmitThreads, 0, st>>>(bins, n, sums);
+    else k_bin_sums<kEmitRounds><<<nb, kEmitThreads, 0, st>>>(bins, n, sums);
     k_scan_spine<<<1, kScanThreads, 0, st>>>(sums, nb, host, seq);
     return 2;
 }
@@ -708,8 +795,13 @@ int launch_emit_pairs_scan(uint32_t n_splats, const uint32_t *order, const uint3
                            const uint32_t *sums, const float4 *rec, int tiles_x, uint32_t n_tiles, uint16_t *ptile,
                            uint32_t *pval, uint2 *ranges, int32_t *blend_meta, cudaStream_t st) {
     if (n_splats == 0) return 0;
-    k_emit_pairs_scan<<<(uint32_t)bin_scan_blocks(n_splats), kScanThreads, 0, st>>>(
-        n_splats, order, bins_sorted, sums, rec, tiles_x, n_tiles, ptile, pval, ranges, blend_meta);
+    const uint32_t nb = (uint32_t)bin_scan_blocks(n_splats);
+    if (n_splats <= kEmitFewSplats)
+        k_emit_pairs_scan<kEmitFewRounds><<<nb, kEmitThreads, 0, st>>>(n_splats, order, bins_sorted, sums, rec, tiles_x,
+                                                                      n_tiles, ptile, pval, ranges, blend_meta);
+    else
+        k_emit_pairs_scan<kEmitRounds><<<nb, kEmitThreads, 0, st>>>(n_splats, order, bins_sorted, sums, rec, tiles_x,
+                                                                   n_tiles, ptile, pval, ranges, blend_meta);
     return 1;
 }
 
