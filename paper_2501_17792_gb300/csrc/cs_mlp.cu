@@ -1,10 +1,10 @@
 // The LoD ranking MLP: 48 -> 64 -> 64 -> 1 with ReLU, BF16 tensor-core
-// matrix products (mma m16n8k16, FP32 accumulate), FP32 master weights and
-// Adam.  One fused kernel runs the forward pass (and, when training, the
-// backward pass with per-CTA weight-gradient partials); a second kernel
-// reduces the partials in a fixed order and applies Adam.
+// matrix products with FP32 accumulation, FP32 master weights and Adam.
+// k_mlp is the forward pass (mma m16n8k16); k_mlp_train a training step's
+// forward and backward pass with per-CTA weight-gradient partials (tcgen05);
+// a third kernel reduces the partials in a fixed order and applies Adam.
 //
-// Warp-level fragments of mma.m16n8k16 (bf16 in, f32 accumulate), lane =
+// Forward pass, warp-level fragments of mma.m16n8k16 (bf16 in, f32 accumulate), lane =
 // 4 * g + q (g = lane / 4, q = lane % 4):
 //   A 16x16 row-major, 4 registers of two bf16 each (low half = lower column):
 //     a0 = A[g][2q, 2q+1]  a1 = A[g+8][2q, 2q+1]  a2 = A[g][2q+8, 2q+9]  a3 = A[g+8][2q+8, 2q+9]
@@ -37,22 +37,15 @@ constexpr int kP = CS_MLP_PARAMS;   // 7361
 constexpr int oW1 = 0, oB1 = oW1 + kIn * kH, oW2 = oB1 + kH, oB2 = oW2 + kH * kH, oW3 = oB2 + kH, oB3 = oW3 + kH;
 static_assert(oB3 + 1 == kP, "parameter layout");
 
-// Warps of a CTA, 16 rows of its tile each.  Training: 12 warps of at most 168
-// registers, one CTA per SM, which hold a thread's 72 gradient sums; the
-// forward pass alone needs half of them.
-__host__ __device__ constexpr int mlp_warps(bool train) { return train ? 12 : 8; }
-__host__ __device__ constexpr int mlp_tile(bool train) { return 16 * mlp_warps(train); }
-// shared-memory leading dimensions (bf16 elements): 28 and 36 words, so that
-// the eight 16-byte rows of an ldmatrix and the 32 words of a fragment store
-// fall in different banks
+// forward pass: 8 warps, 16 rows of the CTA's tile each
+constexpr int kWarps = 8, kThreads = 32 * kWarps, kTile = 16 * kWarps;
+// leading dimensions of the weight copies (bf16 elements): 28 and 36 words, so
+// that the eight 16-byte rows of an ldmatrix fall in different banks
 constexpr int kLdW1 = 56;   // W1^T  [64 hidden][48 in]
 constexpr int kLdW2 = 72;   // W2^T and W2 [64][64]
-constexpr int kLdX = 56;    // activations by row: inputs [row][48],
-constexpr int kLdA = 72;    // hidden units [row][64]
 
 constexpr size_t kW1Elems = (size_t)kH * kLdW1, kW2Elems = (size_t)kH * kLdW2;
-constexpr size_t kSmemWeights = (kW1Elems + 2 * kW2Elems) * 2 + (3 * kH + 4) * 4;
-constexpr size_t kSmemTrain = kSmemWeights + (size_t)mlp_tile(true) * (kLdX + 3 * kLdA) * 2 + (3 * kH + 2) * mlp_warps(true) * 4;
+constexpr size_t kSmemWeights = (kW1Elems + kW2Elems) * 2 + (3 * kH + 4) * 4;
 
 struct Weights {
     const __nv_bfloat16 *w1t;  // [64][kLdW1]: w1t[n][k] = bf16(W1[k][n])
@@ -71,24 +64,17 @@ __device__ __forceinline__ void mma16816(float d[4], const uint32_t a[4], uint32
 
 __device__ __forceinline__ uint32_t bits16(__nv_bfloat16 v) { return (uint32_t)__bfloat16_as_ushort(v); }
 __device__ __forceinline__ uint32_t pack2(__nv_bfloat16 lo, __nv_bfloat16 hi) { return bits16(lo) | (bits16(hi) << 16); }
-__device__ __forceinline__ void st32(__nv_bfloat16 *p, uint32_t v) { *reinterpret_cast<uint32_t *>(p) = v; }
 
 // Four 8x8 bf16 matrices (rows of 16 bytes at the lanes' addresses, lanes 8 i
-// to 8 i + 7 giving matrix i); trans: each transposed.
+// to 8 i + 7 giving matrix i).
 __device__ __forceinline__ void ldsm4(uint32_t r[4], const __nv_bfloat16 *p) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                  : "r"((uint32_t)__cvta_generic_to_shared(p))
                  : "memory");
 }
-__device__ __forceinline__ void ldsm4t(uint32_t r[4], const __nv_bfloat16 *p) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"((uint32_t)__cvta_generic_to_shared(p))
-                 : "memory");
-}
 
-constexpr int kChains = 2;  // independent products in flight: column tiles computed at a time (4: 545 us against 541)
+constexpr int kChains = 2;  // independent products in flight: column tiles computed at a time
 
 // d[i] += a (16 rows x 64) times column tile i of a weight matrix in shared
 // memory; wp: row mr of the first tile, column 8 mi.
@@ -106,16 +92,14 @@ __device__ __forceinline__ void mma_chains(float (&d)[kChains][4], const uint32_
 }
 
 // What a lane reads of its rows g and g + 8: features 8 i + 2 q and the next
-// (i = 0 to 3), the band (-1: none, an all-zero one-hot) and the target.
+// (i = 0 to 3) and the band (-1: none, an all-zero one-hot).
 struct RowInputs {
     float2 x[2][4];
     int band[2];
-    float target[2];
 };
 
-template <bool kTrain>
 __device__ __forceinline__ void load_rows(RowInputs &in, int64_t row, int64_t n, int q, const float *__restrict__ feat,
-                                          const int32_t *__restrict__ band, const float *__restrict__ target) {
+                                          const int32_t *__restrict__ band) {
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int64_t r = row + 8 * h;
@@ -124,51 +108,29 @@ __device__ __forceinline__ void load_rows(RowInputs &in, int64_t row, int64_t n,
         for (int i = 0; i < 4; ++i)
             in.x[h][i] = v ? __ldg(reinterpret_cast<const float2 *>(feat + r * kFeat + 8 * i + 2 * q)) : make_float2(0.f, 0.f);
         in.band[h] = v ? __ldg(band + r) : -1;
-        if (kTrain) in.target[h] = v ? __ldg(target + r) : 0.f;
     }
 }
 
-// Bound by the latency of its shared-memory loads and products at twelve
-// warps an SM: every fragment of the weights and, in training, of the
-// activations comes from shared memory, four 8x8 matrices per ldmatrix.
-// Activations are stored by row as packed pairs; the weight gradients read
-// them transposed (ldmatrix.trans), so nothing is stored element by element.
-// A tile's inputs are loaded during the weight gradients of the tile before.
-// A training step of 2,752,512 rows: 716 us with 8 warps, activations stored
-// transposed element by element and 32-bit fragment loads; 680 with ldmatrix
-// and two CTAs of 8 warps (128 registers, spilled sums), 622 with one CTA of
-// 12 warps, 541 with the inputs loaded ahead and two column tiles at a time.
-template <bool kTrain>
-__global__ void __launch_bounds__(32 * mlp_warps(kTrain), kTrain ? 1 : 2)
-    k_mlp(int64_t n, int n_tiles, const float *__restrict__ feat, const int32_t *__restrict__ band,
-          const float *__restrict__ target, Weights W, float inv_n, float *__restrict__ score,
-          float *__restrict__ partial) {
-    constexpr int kWarps = mlp_warps(kTrain), kThreads = 32 * kWarps, kTile = mlp_tile(kTrain);
+// The forward pass: a warp per 16 rows, weights as fragments from shared
+// memory (four 8x8 matrices per ldmatrix), activations in registers from
+// layer to layer, a tile's inputs loaded during the tile before.
+__global__ void __launch_bounds__(kThreads, 2)
+    k_mlp(int64_t n, int n_tiles, const float *__restrict__ feat, const int32_t *__restrict__ band, Weights W,
+          float *__restrict__ score) {
     extern __shared__ __align__(16) unsigned char smem[];
     __nv_bfloat16 *sW1t = reinterpret_cast<__nv_bfloat16 *>(smem);
     __nv_bfloat16 *sW2t = sW1t + kW1Elems;
-    __nv_bfloat16 *sW2n = sW2t + kW2Elems;
-    float *sb1 = reinterpret_cast<float *>(sW2n + kW2Elems);
+    float *sb1 = reinterpret_cast<float *>(sW2t + kW2Elems);
     float *sb2 = sb1 + kH, *sw3 = sb2 + kH, *sb3 = sw3 + kH;
-    __nv_bfloat16 *sX = reinterpret_cast<__nv_bfloat16 *>(sb3 + 4);  // training only
-    __nv_bfloat16 *sH1 = sX + (size_t)kTile * kLdX;
-    __nv_bfloat16 *sD2 = sH1 + (size_t)kTile * kLdA;
-    __nv_bfloat16 *sD1 = sD2 + (size_t)kTile * kLdA;
-    float *sRed = reinterpret_cast<float *>(sD1 + (size_t)kTile * kLdA);  // [3][kWarps][kH] + [2][kWarps]
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, q = lane & 3;
     const int mi = lane >> 3, mr = lane & 7;  // the matrix and row whose address the lane gives an ldmatrix
     {
         const uint4 *s1 = reinterpret_cast<const uint4 *>(W.w1t);
         const uint4 *s2 = reinterpret_cast<const uint4 *>(W.w2t);
-        const uint4 *s3 = reinterpret_cast<const uint4 *>(W.w2n);
-        uint4 *d1 = reinterpret_cast<uint4 *>(sW1t), *d2 = reinterpret_cast<uint4 *>(sW2t),
-              *d3 = reinterpret_cast<uint4 *>(sW2n);
+        uint4 *d1 = reinterpret_cast<uint4 *>(sW1t), *d2 = reinterpret_cast<uint4 *>(sW2t);
         for (int i = tid; i < (int)(kW1Elems / 8); i += kThreads) d1[i] = s1[i];
-        for (int i = tid; i < (int)(kW2Elems / 8); i += kThreads) {
-            d2[i] = s2[i];
-            if (kTrain) d3[i] = s3[i];
-        }
+        for (int i = tid; i < (int)(kW2Elems / 8); i += kThreads) d2[i] = s2[i];
         for (int i = tid; i < kH; i += kThreads) {
             sb1[i] = W.master[oB1 + i];
             sb2[i] = W.master[oB2 + i];
@@ -178,28 +140,12 @@ __global__ void __launch_bounds__(32 * mlp_warps(kTrain), kTrain ? 1 : 2)
     }
     __syncthreads();
 
-    // training accumulators (per thread, columns 8 nt + 2 q + e)
-    float acc_w3[8][2], acc_b2[8][2], acc_b1[8][2];
-    float acc_dw[6][4];  // this warp's tiles of dW2 (warps 0 to 7: four) or dW1 (warps 8 to 11: six)
-    float acc_b3 = 0.f, acc_loss = 0.f;
-    if (kTrain) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-#pragma unroll
-            for (int e = 0; e < 2; ++e) acc_w3[i][e] = acc_b2[i][e] = acc_b1[i][e] = 0.f;
-#pragma unroll
-        for (int i = 0; i < 6; ++i)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) acc_dw[i][e] = 0.f;
-    }
-
     RowInputs in;
-    load_rows<kTrain>(in, (int64_t)blockIdx.x * kTile + warp * 16 + g, n, q, feat, band, target);
+    load_rows(in, (int64_t)blockIdx.x * kTile + warp * 16 + g, n, q, feat, band);
     for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
         const int64_t r0 = (int64_t)tile * kTile + warp * 16;
         const int64_t ra = r0 + g, rb = r0 + g + 8;
         const bool va = ra < n, vb = rb < n;
-        const int la = warp * 16 + g, lb = la + 8;  // rows within the CTA tile
 
         // ---- layer 1: z1 = x W1 + b1 -------------------------------------
         uint32_t a1[3][4];
@@ -216,12 +162,10 @@ __global__ void __launch_bounds__(32 * mlp_warps(kTrain), kTrain ? 1 : 2)
                                             : make_float2(b < 4 && b == in.band[h] ? 1.f : 0.f,
                                                           b < 4 && b + 1 == in.band[h] ? 1.f : 0.f);
                     a1[kk][2 * half + h] = pack2(__float2bfloat16_rn(x.x), __float2bfloat16_rn(x.y));
-                    if (kTrain) st32(sX + (la + 8 * h) * kLdX + c, a1[kk][2 * half + h]);
                 }
             }
         }
         uint32_t a2[4][4];  // bf16 h1 as layer-2 A fragments
-        uint32_t mask1 = 0;
 #pragma unroll
         for (int n0 = 0; n0 < 8; n0 += kChains) {
             float d[kChains][4];
@@ -242,24 +186,15 @@ __global__ void __launch_bounds__(32 * mlp_warps(kTrain), kTrain ? 1 : 2)
             for (int i = 0; i < kChains; ++i) mma16816(d[i], a1[2], bx[i / 2][2 * (i & 1)], bx[i / 2][2 * (i & 1) + 1]);
 #pragma unroll
             for (int i = 0; i < kChains; ++i) {
-                const int nt = n0 + i, col = 8 * nt + 2 * q;
+                const int nt = n0 + i;
                 __nv_bfloat16 h[4];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    if (d[i][e] > 0.f) mask1 |= 1u << (4 * nt + e);
-                    h[e] = __float2bfloat16_rn(fmaxf(d[i][e], 0.f));
-                }
+                for (int e = 0; e < 4; ++e) h[e] = __float2bfloat16_rn(fmaxf(d[i][e], 0.f));
                 a2[nt >> 1][(nt & 1) * 2] = pack2(h[0], h[1]);
                 a2[nt >> 1][(nt & 1) * 2 + 1] = pack2(h[2], h[3]);
-                if (kTrain) {
-                    st32(sH1 + la * kLdA + col, a2[nt >> 1][(nt & 1) * 2]);
-                    st32(sH1 + lb * kLdA + col, a2[nt >> 1][(nt & 1) * 2 + 1]);
-                }
             }
         }
         // ---- layer 2: z2 = h1 W2 + b2; output y = relu(z2) w3 + b3 --------
-        float h2[8][4];
-        uint32_t mask2 = 0;
         float pa = 0.f, pb = 0.f;
 #pragma unroll
         for (int n0 = 0; n0 < 8; n0 += kChains) {
@@ -273,15 +208,9 @@ __global__ void __launch_bounds__(32 * mlp_warps(kTrain), kTrain ? 1 : 2)
             mma_chains(d, a2, sW2t + (8 * n0 + mr) * kLdW2 + 8 * mi);
 #pragma unroll
             for (int i = 0; i < kChains; ++i) {
-                const int nt = n0 + i;
-                const float2 w3 = *reinterpret_cast<const float2 *>(sw3 + 8 * nt + 2 * q);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    if (d[i][e] > 0.f) mask2 |= 1u << (4 * nt + e);
-                    h2[nt][e] = fmaxf(d[i][e], 0.f);
-                }
-                pa += h2[nt][0] * w3.x + h2[nt][1] * w3.y;
-                pb += h2[nt][2] * w3.x + h2[nt][3] * w3.y;
+                const float2 w3 = *reinterpret_cast<const float2 *>(sw3 + 8 * (n0 + i) + 2 * q);
+                pa += fmaxf(d[i][0], 0.f) * w3.x + fmaxf(d[i][1], 0.f) * w3.y;
+                pb += fmaxf(d[i][2], 0.f) * w3.x + fmaxf(d[i][3], 0.f) * w3.y;
             }
         }
         pa += __shfl_xor_sync(0xffffffffu, pa, 1);
@@ -289,187 +218,554 @@ __global__ void __launch_bounds__(32 * mlp_warps(kTrain), kTrain ? 1 : 2)
         pb += __shfl_xor_sync(0xffffffffu, pb, 1);
         pb += __shfl_xor_sync(0xffffffffu, pb, 2);
         const float ya = pa + sb3[0], yb = pb + sb3[0];
-        if (!kTrain) {
-            if (q == 0) {
-                if (va) score[ra] = ya;
-                if (vb) score[rb] = yb;
-            }
-            load_rows<kTrain>(in, ra + (int64_t)gridDim.x * kTile, n, q, feat, band, target);
-            continue;
-        }
-        // ---- backward ---------------------------------------------------
-        const float ea = va ? ya - in.target[0] : 0.f;
-        const float eb = vb ? yb - in.target[1] : 0.f;
-        const float dya = 2.f * ea * inv_n, dyb = 2.f * eb * inv_n;
         if (q == 0) {
-            acc_loss += ea * ea + eb * eb;
-            acc_b3 += dya + dyb;
+            if (va) score[ra] = ya;
+            if (vb) score[rb] = yb;
         }
-        uint32_t ad[4][4];  // bf16 dz2 as A fragments (k = second hidden unit)
-#pragma unroll
-        for (int nt = 0; nt < 8; ++nt) {
-            const int col = 8 * nt + 2 * q;
-            const float2 w3 = *reinterpret_cast<const float2 *>(sw3 + col);
-            float dz[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const float dy = e < 2 ? dya : dyb;
-                dz[e] = (mask2 >> (4 * nt + e)) & 1u ? dy * (e & 1 ? w3.y : w3.x) : 0.f;
-            }
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                acc_w3[nt][e] += dya * h2[nt][e] + dyb * h2[nt][2 + e];
-                acc_b2[nt][e] += dz[e] + dz[2 + e];
-            }
-            __nv_bfloat16 hb[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) hb[e] = __float2bfloat16_rn(dz[e]);
-            ad[nt >> 1][(nt & 1) * 2] = pack2(hb[0], hb[1]);
-            ad[nt >> 1][(nt & 1) * 2 + 1] = pack2(hb[2], hb[3]);
-            st32(sD2 + la * kLdA + col, ad[nt >> 1][(nt & 1) * 2]);
-            st32(sD2 + lb * kLdA + col, ad[nt >> 1][(nt & 1) * 2 + 1]);
-        }
-        // dh1 = dz2 W2^T, dz1 = dh1 * [z1 > 0]
-#pragma unroll
-        for (int n0 = 0; n0 < 8; n0 += kChains) {
-            float d[kChains][4];
-#pragma unroll
-            for (int i = 0; i < kChains; ++i) d[i][0] = d[i][1] = d[i][2] = d[i][3] = 0.f;
-            mma_chains(d, ad, sW2n + (8 * n0 + mr) * kLdW2 + 8 * mi);
-#pragma unroll
-            for (int i = 0; i < kChains; ++i) {
-                const int nt = n0 + i, col = 8 * nt + 2 * q;
-                __nv_bfloat16 hb[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const float dz = (mask1 >> (4 * nt + e)) & 1u ? d[i][e] : 0.f;
-                    acc_b1[nt][e & 1] += dz;
-                    hb[e] = __float2bfloat16_rn(dz);
-                }
-                st32(sD1 + la * kLdA + col, pack2(hb[0], hb[1]));
-                st32(sD1 + lb * kLdA + col, pack2(hb[2], hb[3]));
-            }
-        }
-        // the next tile's inputs arrive during the weight gradients
-        load_rows<kTrain>(in, ra + (int64_t)gridDim.x * kTile, n, q, feat, band, target);
-        __syncthreads();
-        // ---- weight gradients over the tile's rows ----------------------
-        // Fragments from the row-major tiles, transposed: A (features m, rows
-        // k) matrix i at rows 8 (i / 2), features 8 (i % 2); B (rows k,
-        // features n of two tiles) matrix i at rows 8 (i % 2), features 8 (i / 2)
-        if (warp < 8) {
-            // dW2[m][n] = sum_r h1[r][m] dz2[r][n]: m tile warp/2, n tiles 4 (warp%2) + i
-            const __nv_bfloat16 *ah = sH1 + (8 * (mi >> 1) + mr) * kLdA + 16 * (warp >> 1) + 8 * (mi & 1);
-            const __nv_bfloat16 *bd = sD2 + (8 * (mi & 1) + mr) * kLdA + 32 * (warp & 1) + 8 * (mi >> 1);
-#pragma unroll 4
-            for (int ks = 0; ks < kTile / 16; ++ks) {
-                uint32_t a[4], b[4];
-                ldsm4t(a, ah + 16 * ks * kLdA);
-#pragma unroll
-                for (int i = 0; i < 4; i += 2) {
-                    ldsm4t(b, bd + 16 * ks * kLdA + 8 * i);
-                    mma16816(acc_dw[i], a, b[0], b[1]);
-                    mma16816(acc_dw[i + 1], a, b[2], b[3]);
-                }
-            }
-        } else {
-            // dW1[m][n] = sum_r x[r][m] dz1[r][n]: n tiles 2 (warp - 8) + i, m tiles 0 to 2
-            const __nv_bfloat16 *ax = sX + (8 * (mi >> 1) + mr) * kLdX + 8 * (mi & 1);
-            const __nv_bfloat16 *bz = sD1 + (8 * (mi & 1) + mr) * kLdA + 16 * (warp - 8) + 8 * (mi >> 1);
-#pragma unroll 4
-            for (int ks = 0; ks < kTile / 16; ++ks) {
-                uint32_t a[4], b[4];
-                ldsm4t(b, bz + 16 * ks * kLdA);
-#pragma unroll
-                for (int i = 0; i < 3; ++i) {
-                    ldsm4t(a, ax + 16 * ks * kLdX + 16 * i);
-                    mma16816(acc_dw[2 * i], a, b[0], b[1]);
-                    mma16816(acc_dw[2 * i + 1], a, b[2], b[3]);
-                }
-            }
-        }
-        __syncthreads();  // the activations are rewritten by the next tile
+        load_rows(in, ra + (int64_t)gridDim.x * kTile, n, q, feat, band);
     }
-    if (!kTrain) return;
+}
+
+// ---------------------------------------------------------------------------
+// training: forward, backward and weight gradients on the fifth-generation
+// tensor cores (tcgen05, accumulators in TMEM)
+//
+// A CTA is two groups of eight warps; a group works through tiles of 128 rows
+// by itself, two threads per row (the TMEM lane of the accumulators), one for
+// each half of the 64 hidden units:
+//   Z1 = X W1        M 128, N 64, K 48     then h1 = relu(Z1 + b1)
+//   Z2 = H1 W2       M 128, N 64, K 64     then y, dy, dz2 = dy w3 [z2 > 0]
+//   dH1 = dZ2 W2^T   M 128, N 64, K 64     then dz1 = dH1 [h1 > 0]
+//   G += [H1 | X]^T [dZ2 | dZ1]   M 128, N 128, K 128 (the rows)
+// The last product holds dW2 in its first 64 rows and columns and dW1 in its
+// last; the other two quarters are not read.  It stays in TMEM over all the
+// group's tiles.  The column sums (dw3, db2, db1) stay in registers: 96 per
+// thread, since a thread sees 32 columns of every tile.
+//
+// Activations lie in shared memory row by row, 128 bytes a row, in the
+// 128-byte swizzle (16-byte chunk c of row r at chunk c ^ (r & 7)).  The same
+// bytes serve as a K-major operand (rows are M or N, 8-row groups 1,024 bytes
+// apart) and as an MN-major one (rows are K; the next 64 columns of M or N
+// are in the next buffer), so nothing is transposed.  X has two buffers: the
+// next tile's features arrive by one bulk copy and are converted while a
+// product of this tile runs, and its first product is issued right after this
+// tile's last.  One thread of a group issues all its products, which complete in
+// order, so the wait for one also covers those before it.
+//
+// Bound by latency (issue slots 45%, shared-memory and TMEM data path 47%,
+// tensor pipe 17%): a group's three waits per tile and its loads from TMEM,
+// with two groups an SM, which shared memory (100 KB each) and TMEM (192
+// columns each) allow.  A training step of 2,752,512 rows: 541 us with
+// mma.sync (weights, activations and gradients as fragments from shared
+// memory, 503 us of it this kernel) -> 412 us (372).  One thread per row
+// instead of two 429; the features by 8-byte cp.async 432; FP32 operations
+// one by one and BF16 conversions one by one 466.
+// ---------------------------------------------------------------------------
+
+constexpr int kTcGroups = 2, kTcGroupThreads = 256, kTcThreads = kTcGroupThreads * kTcGroups, kTcRows = 128;
+constexpr uint32_t kTcBuf = kTcRows * 128;            // a buffer of 128 rows
+constexpr uint32_t kTcGroupBytes = 5 * kTcBuf;        // H1, X (two), dZ2, dZ1
+constexpr uint32_t kTcWBuf = kH * 128;                // a weight matrix of 64 rows
+constexpr uint32_t kTcStage = kTcRows * (kFeat + 2) * 4;  // a tile's FP32 features; shares of y
+constexpr uint32_t kTcOffW = kTcGroups * kTcGroupBytes;
+constexpr uint32_t kTcOffStage = kTcOffW + 3 * kTcWBuf;
+static_assert(kTcStage % 128 == 0, "alignment of what follows");
+constexpr uint32_t kTcOffVec = kTcOffStage + kTcGroups * kTcStage;  // b1, b2, w3, b3
+constexpr uint32_t kTcOffBar = kTcOffVec + (3 * kH + 4) * 4;        // mbarriers, TMEM address, fail flags
+constexpr size_t kSmemTc = kTcOffBar + 64 + 1024;                   // (1,024: alignment)
+static_assert(kSmemTc <= 227 * 1024, "shared memory of the training kernel");
+constexpr uint32_t kTcCols = 512;  // TMEM columns: 64 per group for Z, 128 per group for G (from 128 on)
+constexpr long long kTcWaitClocks = 4000000000ll;  // a wait gives up after about two seconds
+
+// matrix descriptor (128-byte swizzle): start address, stride between the
+// 64-column halves of an MN-major operand, 1,024 bytes between 8-row groups
+__device__ __forceinline__ uint64_t tc_desc(uint32_t addr, uint32_t half_stride) {
+    return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)(half_stride >> 4) << 16) | ((uint64_t)(1024u >> 4) << 32) |
+           (1ull << 46) | (2ull << 61);
+}
+// instruction descriptor: BF16 operands, FP32 accumulator
+__host__ __device__ constexpr uint32_t tc_idesc(bool mn_major, int m, int n) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((mn_major ? 3u : 0u) << 15) | ((uint32_t)(n / 8) << 17) |
+           ((uint32_t)(m / 16) << 24);
+}
+
+__device__ __forceinline__ void tc_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, bool accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"((uint32_t)accumulate)
+        : "memory");
+}
+// the mbarrier arrives when all products issued so far by this thread are done
+__device__ __forceinline__ void tc_commit(uint32_t bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tc_fence_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+__device__ __forceinline__ void group_sync(int group) { asm volatile("bar.sync %0, 256;" ::"r"(group + 1) : "memory"); }
+
+// Waits for phase `parity` of the mbarrier; false after kTcWaitClocks.
+__device__ __forceinline__ bool tc_wait(uint32_t bar, uint32_t parity) {
+    const long long t0 = clock64();
+    for (;;) {
+        uint32_t done;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(done)
+            : "r"(bar), "r"(parity)
+            : "memory");
+        if (done) return true;
+        if (clock64() - t0 > kTcWaitClocks) return false;
+    }
+}
+
+// pairs of FP32 values, one instruction for both
+using f2 = unsigned long long;
+__device__ __forceinline__ f2 make2(float lo, float hi) {
+    return (f2)__float_as_uint(lo) | ((f2)__float_as_uint(hi) << 32);
+}
+__device__ __forceinline__ float lo2(f2 v) { return __uint_as_float((uint32_t)v); }
+__device__ __forceinline__ float hi2(f2 v) { return __uint_as_float((uint32_t)(v >> 32)); }
+__device__ __forceinline__ f2 add2(f2 a, f2 b) {
+    f2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
+    f2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+    f2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ f2 relu2(f2 v) { return make2(fmaxf(lo2(v), 0.f), fmaxf(hi2(v), 0.f)); }
+
+// sixteen columns of the thread's TMEM lane, in pairs
+__device__ __forceinline__ void tc_load16(f2 (&z)[8], uint32_t addr) {
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(addr)
+        : "memory");
+#pragma unroll
+    for (int i = 0; i < 8; ++i) z[i] = (f2)r[2 * i] | ((f2)r[2 * i + 1] << 32);
+}
+
+__device__ __forceinline__ uint32_t cvt2(f2 v) {  // to two BF16, the lower in the lower half
+    const __nv_bfloat162 h = __floats2bfloat162_rn(lo2(v), hi2(v));
+    return *reinterpret_cast<const uint32_t *>(&h);
+}
+// 16-byte chunk c of row r of a swizzled buffer
+__device__ __forceinline__ uint4 *tc_chunk(unsigned char *buf, int r, int c) {
+    return reinterpret_cast<uint4 *>(buf + r * 128 + ((c ^ (r & 7)) << 4));
+}
+
+// The tile's FP32 features to the staging buffer: one bulk copy, whose
+// arrival the mbarrier counts, or (an array at an odd multiple of 8 bytes)
+// loads and stores by the group's threads.  t: thread of the group.
+__device__ __forceinline__ void tc_stage(unsigned char *stage, uint32_t bar, bool bulk, int64_t row0, int64_t n, int t,
+                                         const float *__restrict__ feat) {
+    const int rows = (int)min((int64_t)kTcRows, n - row0);
+    const float *src = feat + row0 * kFeat;
+    if (!bulk) {
+        for (int i = t; i < rows * kFeat / 2; i += kTcGroupThreads)
+            reinterpret_cast<float2 *>(stage)[i] = __ldg(reinterpret_cast<const float2 *>(src) + i);
+    } else if (t == 32) {
+        const uint32_t bytes = (uint32_t)rows * kFeat * 4;
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                         (uint32_t)__cvta_generic_to_shared(stage)),
+                     "l"(src), "r"(bytes), "r"(bar)
+                     : "memory");
+    }
+}
+
+// The staged features to X as BF16, and by the first half's threads their
+// row's one-hot band (columns 40 to 63 stay zero); rows past n are zero.
+__device__ __forceinline__ void tc_input(unsigned char *x, const unsigned char *stage, int64_t row0, int64_t n, int t,
+                                         int band) {
+    const int r0 = t >> 3, p = t & 7;  // 16-byte piece p of rows r0 + 32 i
+    unsigned char *to = x + r0 * 128 + (((p >> 1) ^ (r0 & 7)) << 4) + 8 * (p & 1);
+#pragma unroll
+    for (int i = 0; i < kTcRows / 32; ++i) {
+        float4 a = reinterpret_cast<const float4 *>(stage)[t + kTcGroupThreads * i];
+        if (row0 + r0 + 32 * i >= n) a = make_float4(0.f, 0.f, 0.f, 0.f);
+        *reinterpret_cast<uint2 *>(to + 4096 * i) = make_uint2(cvt2(make2(a.x, a.y)), cvt2(make2(a.z, a.w)));
+    }
+    if (t < kTcRows) {
+        const uint32_t one = 0x3F80u;  // 1.0
+        *tc_chunk(x, t, 4) = make_uint4((band == 0 ? one : 0u) | (band == 1 ? one << 16 : 0u),
+                                        (band == 2 ? one : 0u) | (band == 3 ? one << 16 : 0u), 0u, 0u);
+    }
+}
+
+__global__ void __launch_bounds__(kTcThreads, 1)
+    k_mlp_train(int64_t n, int n_tiles, const float *__restrict__ feat, const int32_t *__restrict__ band,
+                const float *__restrict__ target, Weights W, float inv_n, bool bulk, float *__restrict__ partial,
+                uint32_t *__restrict__ err) {
+    extern __shared__ unsigned char tc_raw[];
+    unsigned char *smem = tc_raw + ((1024u - ((uint32_t)__cvta_generic_to_shared(tc_raw) & 1023u)) & 1023u);
+    // t: thread of the group; r: its row of the tile, half: its half of the hidden units
+    const int tid = threadIdx.x, group = tid >> 8, t = tid & 255, half = t >> 7, r = t & 127, warp = tid >> 5, lane = tid & 31;
+    unsigned char *sH1 = smem + group * kTcGroupBytes, *sX = sH1 + kTcBuf, *sD2 = sX + 2 * kTcBuf, *sD1 = sD2 + kTcBuf;
+    unsigned char *sW = smem + kTcOffW;  // W1^T, W2^T, W2
+    unsigned char *stage = smem + kTcOffStage + group * kTcStage;
+    float *s_y = reinterpret_cast<float *>(stage) + kTcRows * kFeat;  // shares of y, by half
+    float *sb1 = reinterpret_cast<float *>(smem + kTcOffVec), *sb2 = sb1 + kH, *sw3 = sb2 + kH, *sb3 = sw3 + kH;
+    const ulonglong2 *vb1 = reinterpret_cast<const ulonglong2 *>(sb1), *vb2 = reinterpret_cast<const ulonglong2 *>(sb2),
+                     *vw3 = reinterpret_cast<const ulonglong2 *>(sw3);  // four values each
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kTcOffBar);
+    uint32_t *s_tmem = reinterpret_cast<uint32_t *>(bars + 2 * kTcGroups);
+    volatile uint32_t *s_fail = s_tmem + 1;  // per group
+    // of a group: its products, its staged features
+    const uint32_t bar = (uint32_t)__cvta_generic_to_shared(bars + group), stage_bar = bar + 8 * kTcGroups;
+
+    // weights into the swizzled layout (columns past a row's length zero)
+    for (int i = tid; i < 3 * kH * 8; i += kTcThreads) {
+        const int m = i / (kH * 8), wr = (i >> 3) & (kH - 1), c = i & 7;
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (m == 0) {
+            if (c < kIn / 8) v = *reinterpret_cast<const uint4 *>(W.w1t + wr * kLdW1 + 8 * c);
+        } else {
+            v = *reinterpret_cast<const uint4 *>((m == 1 ? W.w2t : W.w2n) + wr * kLdW2 + 8 * c);
+        }
+        *tc_chunk(sW + m * kTcWBuf, wr, c) = v;
+    }
+    for (int i = tid; i < kH; i += kTcThreads) {
+        sb1[i] = W.master[oB1 + i];
+        sb2[i] = W.master[oB2 + i];
+        sw3[i] = W.master[oW3 + i];
+    }
+    for (int c = 5; c < 8; ++c) *tc_chunk(sX + half * kTcBuf, r, c) = make_uint4(0u, 0u, 0u, 0u);
+    if (tid == 0) {
+        sb3[0] = W.master[oB3];
+        for (int g = 0; g < 2 * kTcGroups; ++g)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((uint32_t)__cvta_generic_to_shared(bars + g)) : "memory");
+        for (int g = 0; g < kTcGroups; ++g) s_fail[g] = 0u;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        __syncwarp();
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                         (uint32_t)__cvta_generic_to_shared(s_tmem)),
+                     "r"(kTcCols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_smem();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *s_tmem;
+    const uint32_t z_cols = tmem + 64u * group, g_cols = tmem + 128u + 128u * group;
+    const uint32_t my_lanes = (uint32_t)(warp & 3) << 21;  // lane 32 (warp % 4) in bits 16 and up
+    constexpr int kMine = kH / 2;                          // the thread's columns, from `mine` on
+    const int mine = kMine * half;
+    const bool issuer = t == 0;
+    const uint32_t aH1 = (uint32_t)__cvta_generic_to_shared(sH1), aX = (uint32_t)__cvta_generic_to_shared(sX),
+                   aD2 = (uint32_t)__cvta_generic_to_shared(sD2), aW = (uint32_t)__cvta_generic_to_shared(sW);
+    constexpr uint32_t kFwd = tc_idesc(false, 128, 64), kGrad = tc_idesc(true, 128, 128);
+
+    f2 s_w3[kMine / 2], s_b2[kMine / 2], s_b1[kMine / 2];  // column sums over the thread's rows
+#pragma unroll
+    for (int i = 0; i < kMine / 2; ++i) s_w3[i] = s_b2[i] = s_b1[i] = 0ull;
+    float acc_loss = 0.f, acc_b3 = 0.f;
+    uint32_t phase = 0;
+    bool any = false;  // a tile has been added to G
+    const int first = (int)blockIdx.x * kTcGroups + group, step = (int)gridDim.x * kTcGroups;
+
+    // the first tile's inputs and first product
+    int nband = -1;
+    float ntarget = 0.f;
+    uint32_t stage_phase = 0;
+    auto next_row = [&](int64_t row) {  // band and target of the thread's row of a coming tile
+        nband = row < n ? __ldg(band + row) : -1;
+        ntarget = row < n ? __ldg(target + row) : 0.f;
+    };
+    auto staged = [&] {  // the staged features are there
+        if (!bulk) {
+            group_sync(group);
+        } else {
+            if (!tc_wait(stage_bar, stage_phase)) s_fail[group] = 1u;
+            stage_phase ^= 1u;
+        }
+    };
+    if (first < n_tiles) {
+        const int64_t row0 = (int64_t)first * kTcRows;
+        tc_stage(stage, stage_bar, bulk, row0, n, t, feat);
+        next_row(row0 + r);
+        staged();
+        tc_input(sX, stage, row0, n, t, nband);
+        tc_fence_smem();
+        tc_fence_before();
+        group_sync(group);
+        if (first + step < n_tiles) tc_stage(stage, stage_bar, bulk, (int64_t)(first + step) * kTcRows, n, t, feat);
+        if (issuer) {
+            tc_fence_after();
+#pragma unroll
+            for (int k = 0; k < kIn / 16; ++k) tc_mma(z_cols, tc_desc(aX + 32 * k, 0), tc_desc(aW + 32 * k, 0), kFwd, k > 0);
+            tc_commit(bar);
+        }
+    }
+    int xbuf = 0;
+    bool staging = first + step < n_tiles;  // a copy may be in flight
+    for (int tile = first; tile < n_tiles; tile += step, xbuf ^= 1) {
+        const bool valid = (int64_t)tile * kTcRows + r < n, more = tile + step < n_tiles;
+        const int64_t next0 = (int64_t)(tile + step) * kTcRows;
+        const float y_target = ntarget;
+        if (more) next_row(next0 + r);
+        // ---- h1 = relu(Z1 + b1) ------------------------------------------
+        if (!tc_wait(bar, phase)) s_fail[group] = 1u;
+        phase ^= 1u;
+        __syncwarp();
+        tc_fence_after();
+#pragma unroll
+        for (int c0 = 0; c0 < kMine; c0 += 16) {
+            f2 z[8];
+            tc_load16(z, z_cols + my_lanes + mine + c0);
+            uint32_t h[8];
+#pragma unroll
+            for (int i = 0; i < 8; i += 2) {
+                const ulonglong2 b = vb1[(mine + c0) / 4 + i / 2];
+                h[i] = cvt2(relu2(add2(z[i], b.x)));
+                h[i + 1] = cvt2(relu2(add2(z[i + 1], b.y)));
+            }
+            *tc_chunk(sH1, r, (mine + c0) / 8) = make_uint4(h[0], h[1], h[2], h[3]);
+            *tc_chunk(sH1, r, (mine + c0) / 8 + 1) = make_uint4(h[4], h[5], h[6], h[7]);
+        }
+        tc_fence_smem();
+        tc_fence_before();
+        group_sync(group);
+        if (s_fail[group]) break;  // the same for the whole group: set before the barrier
+        if (issuer) {
+            tc_fence_after();
+#pragma unroll
+            for (int k = 0; k < kH / 16; ++k)
+                tc_mma(z_cols, tc_desc(aH1 + 32 * k, 0), tc_desc(aW + kTcWBuf + 32 * k, 0), kFwd, k > 0);
+            tc_commit(bar);
+        }
+        // the next tile's inputs, while Z2 is computed
+        if (more) {
+            staged();
+            staging = false;
+            tc_input(sX + (xbuf ^ 1) * kTcBuf, stage, next0, n, t, nband);
+        }
+        // ---- y, dy, dz2 = dy w3 [z2 > 0] ---------------------------------
+        if (!tc_wait(bar, phase)) s_fail[group] = 1u;
+        phase ^= 1u;
+        __syncwarp();
+        tc_fence_after();
+        f2 y2 = 0ull;
+#pragma unroll
+        for (int c0 = 0; c0 < kMine; c0 += 16) {
+            f2 z[8];
+            tc_load16(z, z_cols + my_lanes + mine + c0);
+#pragma unroll
+            for (int i = 0; i < 8; i += 2) {
+                const ulonglong2 b = vb2[(mine + c0) / 4 + i / 2], w = vw3[(mine + c0) / 4 + i / 2];
+                y2 = fma2(relu2(add2(z[i], b.x)), w.x, y2);
+                y2 = fma2(relu2(add2(z[i + 1], b.y)), w.y, y2);
+            }
+        }
+        // the halves' shares of y meet in shared memory
+        s_y[t] = lo2(y2) + hi2(y2);
+        group_sync(group);
+        const float y = s_y[r] + s_y[r + 128];
+        const float e = valid ? y + sb3[0] - y_target : 0.f;
+        const float dy = 2.f * e * inv_n;
+        const f2 dy2 = make2(dy, dy);
+        if (half == 0) {
+            acc_loss += e * e;
+            acc_b3 += dy;
+        }
+#pragma unroll
+        for (int c0 = 0; c0 < kMine; c0 += 16) {
+            f2 z[8];
+            tc_load16(z, z_cols + my_lanes + mine + c0);
+            uint32_t h[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const ulonglong2 b4 = vb2[(mine + c0) / 4 + i / 2], w4 = vw3[(mine + c0) / 4 + i / 2];
+                const f2 zb = add2(z[i], i & 1 ? b4.y : b4.x), p = mul2(dy2, i & 1 ? w4.y : w4.x);
+                const f2 d = make2(lo2(zb) > 0.f ? lo2(p) : 0.f, hi2(zb) > 0.f ? hi2(p) : 0.f);
+                s_w3[c0 / 2 + i] = fma2(dy2, relu2(zb), s_w3[c0 / 2 + i]);
+                s_b2[c0 / 2 + i] = add2(s_b2[c0 / 2 + i], d);
+                h[i] = cvt2(d);
+            }
+            *tc_chunk(sD2, r, (mine + c0) / 8) = make_uint4(h[0], h[1], h[2], h[3]);
+            *tc_chunk(sD2, r, (mine + c0) / 8 + 1) = make_uint4(h[4], h[5], h[6], h[7]);
+        }
+        tc_fence_smem();
+        tc_fence_before();
+        group_sync(group);
+        if (s_fail[group]) break;
+        staging = tile + 2 * step < n_tiles;
+        if (staging) tc_stage(stage, stage_bar, bulk, (int64_t)(tile + 2 * step) * kTcRows, n, t, feat);
+        if (issuer) {
+            tc_fence_after();
+#pragma unroll
+            for (int k = 0; k < kH / 16; ++k)
+                tc_mma(z_cols, tc_desc(aD2 + 32 * k, 0), tc_desc(aW + 2 * kTcWBuf + 32 * k, 0), kFwd, k > 0);
+            tc_commit(bar);
+        }
+        // ---- dz1 = dH1 [h1 > 0] ------------------------------------------
+        if (!tc_wait(bar, phase)) s_fail[group] = 1u;
+        phase ^= 1u;
+        __syncwarp();
+        tc_fence_after();
+#pragma unroll
+        for (int c0 = 0; c0 < kMine; c0 += 16) {
+            f2 z[8];
+            tc_load16(z, z_cols + my_lanes + mine + c0);
+            const uint4 ha = *tc_chunk(sH1, r, (mine + c0) / 8), hb = *tc_chunk(sH1, r, (mine + c0) / 8 + 1);
+            const uint32_t hw[8] = {ha.x, ha.y, ha.z, ha.w, hb.x, hb.y, hb.z, hb.w};
+            uint32_t h[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const f2 d = make2(hw[i] & 0xFFFFu ? lo2(z[i]) : 0.f, hw[i] > 0xFFFFu ? hi2(z[i]) : 0.f);
+                s_b1[c0 / 2 + i] = add2(s_b1[c0 / 2 + i], d);
+                h[i] = cvt2(d);
+            }
+            *tc_chunk(sD1, r, (mine + c0) / 8) = make_uint4(h[0], h[1], h[2], h[3]);
+            *tc_chunk(sD1, r, (mine + c0) / 8 + 1) = make_uint4(h[4], h[5], h[6], h[7]);
+        }
+        tc_fence_smem();
+        tc_fence_before();
+        group_sync(group);
+        if (s_fail[group]) break;
+        if (issuer) {
+            tc_fence_after();
+            // G, sixteen rows a product: [H1 | X] and [dZ2 | dZ1]
+            const uint32_t to_x = kTcBuf * (1 + xbuf);
+#pragma unroll
+            for (int k = 0; k < kTcRows / 16; ++k)
+                tc_mma(g_cols, tc_desc(aH1 + 2048 * k, to_x), tc_desc(aD2 + 2048 * k, kTcBuf), kGrad, any || k > 0);
+            if (more) {
+                const uint32_t x = aX + (xbuf ^ 1) * kTcBuf;
+#pragma unroll
+                for (int k = 0; k < kIn / 16; ++k) tc_mma(z_cols, tc_desc(x + 32 * k, 0), tc_desc(aW + 32 * k, 0), kFwd, k > 0);
+            }
+            tc_commit(bar);
+        }
+        any = true;
+    }
+    if (bulk && staging) tc_wait(stage_bar, stage_phase);  // (after a failed wait only)
+    if (any && !s_fail[group] && !tc_wait(bar, phase)) s_fail[group] = 1u;
+    __syncwarp();
+    tc_fence_after();
+    __syncthreads();
 
     // ---- per-CTA partial gradient, written in a fixed order --------------
+    // the groups' G: a row's two threads read half of its columns each; group
+    // 1 leaves its quarters in shared memory (over the activations), group 0
+    // adds them
     float *out = partial + (size_t)blockIdx.x * (kP + 1);
+    constexpr int kLdG = 65;
+    float *sG = reinterpret_cast<float *>(smem);            // [128][kLdG]
+    float *sRed = sG + 128 * kLdG;                          // [8 warp rows][3 kH + 2]
+    constexpr int kLdR = 3 * kH + 2;
+    const uint32_t my_g = g_cols + my_lanes + (r < kH ? 0 : kH) + mine;  // dW2's columns, dW1's
 #pragma unroll
-    for (int i = 0; i < 6; ++i) {
-        // tile i: rows m and m + 8, columns c and c + 1 of W2 or W1
-        if (warp < 8 && i >= 4) break;
-        const int o = warp < 8 ? oW2 : oW1;
-        const int m = 16 * (warp < 8 ? warp >> 1 : i >> 1) + g;
-        const int c = 8 * (warp < 8 ? 4 * (warp & 1) + i : 2 * (warp - 8) + (i & 1)) + 2 * q;
-        out[o + m * kH + c] = acc_dw[i][0];
-        out[o + m * kH + c + 1] = acc_dw[i][1];
-        out[o + (m + 8) * kH + c] = acc_dw[i][2];
-        out[o + (m + 8) * kH + c + 1] = acc_dw[i][3];
-    }
-    // column sums: over the 8 lanes of equal q, then over warps via shared memory
-    float *rw3 = sRed, *rb2 = rw3 + kWarps * kH, *rb1 = rb2 + kWarps * kH, *rs = rb1 + kWarps * kH;
+    for (int c0 = 0; c0 < kMine; c0 += 16) {
+        f2 z[8];
+        // (warps 0, 1, 4 and 5 of a group hold dW2's rows, the others dW1's)
+        tc_load16(z, my_g + c0);
+        if (group == 1) {
 #pragma unroll
-    for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            float a = acc_w3[nt][e], b = acc_b2[nt][e], c = acc_b1[nt][e];
-#pragma unroll
-            for (int s = 4; s < 32; s <<= 1) {
-                a += __shfl_xor_sync(0xffffffffu, a, s);
-                b += __shfl_xor_sync(0xffffffffu, b, s);
-                c += __shfl_xor_sync(0xffffffffu, c, s);
-            }
-            if (g == 0) {
-                const int col = 8 * nt + 2 * q + e;
-                rw3[warp * kH + col] = a;
-                rb2[warp * kH + col] = b;
-                rb1[warp * kH + col] = c;
-            }
+            for (int i = 0; i < 16; ++i) sG[r * kLdG + mine + c0 + i] = any ? (i & 1 ? hi2(z[i / 2]) : lo2(z[i / 2])) : 0.f;
         }
+    }
+    float *red = sRed + (4 * group + (warp & 3)) * kLdR;  // 32 rows of the tiles, both halves' columns
+#pragma unroll
+    for (int i = 0; i < kMine; ++i) {
+        float a = i & 1 ? hi2(s_w3[i / 2]) : lo2(s_w3[i / 2]), b = i & 1 ? hi2(s_b2[i / 2]) : lo2(s_b2[i / 2]),
+              c = i & 1 ? hi2(s_b1[i / 2]) : lo2(s_b1[i / 2]);
+#pragma unroll
+        for (int s = 1; s < 32; s <<= 1) {
+            a += __shfl_xor_sync(0xffffffffu, a, s);
+            b += __shfl_xor_sync(0xffffffffu, b, s);
+            c += __shfl_xor_sync(0xffffffffu, c, s);
+        }
+        if (lane == 0) {
+            red[mine + i] = a;
+            red[kH + mine + i] = b;
+            red[2 * kH + mine + i] = c;
+        }
+    }
     float l = acc_loss, b3 = acc_b3;
 #pragma unroll
     for (int s = 1; s < 32; s <<= 1) {
         l += __shfl_xor_sync(0xffffffffu, l, s);
         b3 += __shfl_xor_sync(0xffffffffu, b3, s);
     }
-    if (lane == 0) {
-        rs[warp] = b3;
-        rs[kWarps + warp] = l;
+    if (lane == 0 && half == 0) {
+        red[3 * kH] = b3;
+        red[3 * kH + 1] = l;
     }
     __syncthreads();
-    if (tid < kH) {
-        float a = 0.f, b = 0.f, c = 0.f;
-        for (int w = 0; w < kWarps; ++w) {
-            a += rw3[w * kH + tid];
-            b += rb2[w * kH + tid];
-            c += rb1[w * kH + tid];
+    if (group == 0) {
+#pragma unroll
+        for (int c0 = 0; c0 < kMine; c0 += 16) {
+            f2 z[8];
+            tc_load16(z, my_g + c0);
+            // row r of dW2, row r - 64 of dW1 (its rows past kIn are padding)
+            if (r < kH + kIn) {
+                float *o = out + (r < kH ? oW2 + r * kH : oW1 + (r - kH) * kH) + mine + c0;
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                    o[i] = (any ? (i & 1 ? hi2(z[i / 2]) : lo2(z[i / 2])) : 0.f) + sG[r * kLdG + mine + c0 + i];
+            }
         }
-        out[oW3 + tid] = a;
-        out[oB2 + tid] = b;
-        out[oB1 + tid] = c;
     }
-    if (tid == 0) {
-        float a = 0.f, b = 0.f;
-        for (int w = 0; w < kWarps; ++w) {
-            a += rs[w];
-            b += rs[kWarps + w];
-        }
-        out[oB3] = a;
-        out[kP] = b;  // sum of squared errors
+    if (tid < kLdR) {
+        float a = 0.f;
+        for (int w = 0; w < 4 * kTcGroups; ++w) a += sRed[w * kLdR + tid];
+        const int o = tid < kH ? oW3 + tid : tid < 2 * kH ? oB2 + tid - kH : tid < 3 * kH ? oB1 + tid - 2 * kH
+                                                                          : tid == 3 * kH ? oB3 : kP;
+        out[o] = a;  // (kP: the sum of squared errors)
+    }
+    if (t == 0 && s_fail[group]) atomicOr(err, 1u);
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcCols) : "memory");
     }
 }
 
-// Sum the per-CTA partials (fixed order), then Adam on the FP32 master
-// weights and refresh the BF16 copies.  One thread per parameter; thread kP
-// sums the squared errors.
-__global__ void k_mlp_adam(int n_part, const float *__restrict__ partial, float *__restrict__ master,
-                           float *__restrict__ m1, float *__restrict__ m2, float *__restrict__ grad,
-                           __nv_bfloat16 *__restrict__ w1t, __nv_bfloat16 *__restrict__ w2t,
-                           __nv_bfloat16 *__restrict__ w2n, float lr, float bc1, float bc2, float *__restrict__ sse) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p > kP) return;
+// Sum the per-CTA partials, then Adam on the FP32 master weights and refresh
+// the BF16 copies.  A block takes 32 parameters, a warp a run of the
+// partials; the eight warps' sums are added in order.  Parameter kP is the
+// sum of the squared errors.  After a training kernel that gave up waiting
+// (*err) the parameters stay as they are.  One thread per parameter over all
+// 152 partials took 16 us (a chain of loads).
+constexpr int kAdamWarps = 8;
+
+__global__ void __launch_bounds__(32 * kAdamWarps)
+    k_mlp_adam(int n_part, const float *__restrict__ partial, float *__restrict__ master, float *__restrict__ m1,
+               float *__restrict__ m2, float *__restrict__ grad, __nv_bfloat16 *__restrict__ w1t,
+               __nv_bfloat16 *__restrict__ w2t, __nv_bfloat16 *__restrict__ w2n, float lr, float bc1, float bc2,
+               float *__restrict__ sse, const uint32_t *__restrict__ err) {
+    __shared__ float sums[kAdamWarps][32];
+    const int warp = threadIdx.x >> 5, p = blockIdx.x * 32 + (threadIdx.x & 31);
+    const int run = (n_part + kAdamWarps - 1) / kAdamWarps, c1 = min(n_part, (warp + 1) * run);
     float s = 0.f;
-    for (int c = 0; c < n_part; ++c) s += partial[(size_t)c * (kP + 1) + p];
+    if (p <= kP) {
+#pragma unroll 8
+        for (int c = warp * run; c < c1; ++c) s += partial[(size_t)c * (kP + 1) + p];
+    }
+    sums[warp][threadIdx.x & 31] = s;
+    __syncthreads();
+    if (warp > 0 || p > kP || *err) return;
+    s = 0.f;
+    for (int w = 0; w < kAdamWarps; ++w) s += sums[w][threadIdx.x];
     if (p == kP) {
         *sse = s;
         return;
@@ -552,9 +848,8 @@ int mfail(cs_mlp *m, int code, const char *fmt, ...) {
 
 bool aligned(const void *p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; }
 
-int grid_for(const cs_mlp *m, int64_t n, bool train) {
-    const int64_t tiles = (n + mlp_tile(train) - 1) / mlp_tile(train);
-    return (int)std::min<int64_t>(tiles, (train ? 1LL : 2LL) * m->n_sm);
+int grid_for(const cs_mlp *m, int64_t n, int rows, int per_sm) {
+    return (int)std::min<int64_t>((n + rows - 1) / rows, (int64_t)per_sm * m->n_sm);
 }
 
 int refresh_copies(cs_mlp *m) {
@@ -590,8 +885,7 @@ int cs_mlp_create(cs_mlp **out, int32_t device, void *stream, uint64_t seed) {
         cudaGetLastError();
         return bail(CS_ERR_OOM);
     }
-    if (cudaFuncSetAttribute(k_mlp<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemTrain) != cudaSuccess ||
-        cudaFuncSetAttribute(k_mlp<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemTrain) != cudaSuccess)
+    if (cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemTc) != cudaSuccess)
         return bail(CS_ERR_CUDA);
     // initial weights from the counter-based generator
     std::vector<float> p(kP, 0.0f);
@@ -646,6 +940,7 @@ int cs_mlp_set_params(cs_mlp *m, const float *host_in) {
     MLP_CUDA(m, cudaMemcpyAsync(m->master, host_in, kP * 4, cudaMemcpyHostToDevice, m->stream));
     MLP_CUDA(m, cudaMemsetAsync(m->m1, 0, kP * 4, m->stream));
     MLP_CUDA(m, cudaMemsetAsync(m->m2, 0, kP * 4, m->stream));
+    MLP_CUDA(m, cudaMemsetAsync(m->sse, 0, 16, m->stream));
     int rc = refresh_copies(m);
     if (rc != CS_OK) return rc;
     MLP_CUDA(m, cudaStreamSynchronize(m->stream));
@@ -661,10 +956,9 @@ int cs_mlp_forward(cs_mlp *m, int64_t n, const float *feat, const int32_t *band,
     if (!feat || !band || !score_out || !aligned(feat, 8) || !aligned(band, 4) || !aligned(score_out, 4))
         return mfail(m, CS_ERR_ARG, "NULL or misaligned array");
     MLP_CUDA(m, cudaSetDevice(m->device));
-    const int tiles = (int)((n + mlp_tile(false) - 1) / mlp_tile(false));
+    const int tiles = (int)((n + kTile - 1) / kTile);
     Weights W{m->w1t, m->w2t, m->w2n, m->master};
-    k_mlp<false><<<grid_for(m, n, false), 32 * mlp_warps(false), kSmemWeights, m->stream>>>(n, tiles, feat, band, nullptr, W, 0.f,
-                                                                       score_out, nullptr);
+    k_mlp<<<grid_for(m, n, kTile, 2), kThreads, kSmemWeights, m->stream>>>(n, tiles, feat, band, W, score_out);
     MLP_CUDA(m, cudaGetLastError());
     return CS_OK;
 }
@@ -678,7 +972,7 @@ int cs_mlp_train_step(cs_mlp *m, int64_t n, const float *feat, const int32_t *ba
     if (!feat || !band || !target || !aligned(feat, 8) || !aligned(band, 4) || !aligned(target, 4))
         return mfail(m, CS_ERR_ARG, "NULL or misaligned array");
     MLP_CUDA(m, cudaSetDevice(m->device));
-    const int grid = grid_for(m, n, true);
+    const int grid = grid_for(m, n, kTcGroups * kTcRows, 1);
     if (grid > m->n_part_cap) {
         MLP_CUDA(m, cudaStreamSynchronize(m->stream));
         cudaFree(m->partial);
@@ -687,20 +981,24 @@ int cs_mlp_train_step(cs_mlp *m, int64_t n, const float *feat, const int32_t *ba
         MLP_CUDA(m, cudaMalloc(&m->partial, (size_t)grid * (kP + 1) * 4));
         m->n_part_cap = grid;
     }
-    const int tiles = (int)((n + mlp_tile(true) - 1) / mlp_tile(true));
+    const int tiles = (int)((n + kTcRows - 1) / kTcRows);
     Weights W{m->w1t, m->w2t, m->w2n, m->master};
-    k_mlp<true><<<grid, 32 * mlp_warps(true), kSmemTrain, m->stream>>>(n, tiles, feat, band, target, W, (float)(1.0 / (double)n),
-                                                          nullptr, m->partial);
+    uint32_t *err = reinterpret_cast<uint32_t *>(m->sse + 1);
+    k_mlp_train<<<grid, kTcThreads, kSmemTc, m->stream>>>(n, tiles, feat, band, target, W, (float)(1.0 / (double)n),
+                                                          aligned(feat, 16), m->partial, err);
     MLP_CUDA(m, cudaGetLastError());
     const int64_t t = m->steps + 1;
     const float bc1 = (float)(1.0 - std::pow(0.9, (double)t)), bc2 = (float)(1.0 - std::pow(0.999, (double)t));
-    k_mlp_adam<<<(kP + 1 + 255) / 256, 256, 0, m->stream>>>(grid, m->partial, m->master, m->m1, m->m2, m->grad,
-                                                              m->w1t, m->w2t, m->w2n, lr, bc1, bc2, m->sse);
+    k_mlp_adam<<<(kP + 1 + 31) / 32, 32 * kAdamWarps, 0, m->stream>>>(grid, m->partial, m->master, m->m1, m->m2, m->grad,
+                                                              m->w1t, m->w2t, m->w2n, lr, bc1, bc2, m->sse, err);
     MLP_CUDA(m, cudaGetLastError());
     m->steps = t;
     if (loss_out) {
-        MLP_CUDA(m, cudaMemcpyAsync(m->h_sse, m->sse, 4, cudaMemcpyDeviceToHost, m->stream));
+        MLP_CUDA(m, cudaMemcpyAsync(m->h_sse, m->sse, 8, cudaMemcpyDeviceToHost, m->stream));
         MLP_CUDA(m, cudaStreamSynchronize(m->stream));
+        uint32_t failed;
+        std::memcpy(&failed, m->h_sse + 1, 4);
+        if (failed) return mfail(m, CS_ERR_CUDA, "the training kernel gave up waiting for its tensor-core products");
         *loss_out = (float)((double)m->h_sse[0] / (double)n);
     }
     return CS_OK;
