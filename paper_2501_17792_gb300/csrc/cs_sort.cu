@@ -381,6 +381,12 @@ __global__ void __launch_bounds__(kRadixThreads, 3) k_radix_scatter(
 // next.  Same digits, same order.  A 256x256 frame of 16,384 splats: 194 ->
 // 162 us; a training frame of 12,291 splats: 424 -> 394 us.
 constexpr int kClusterBlocks = 8;  // the portable cluster size
+// Twice the threads of the pass-by-pass kernels, half the elements each: one
+// block's latency is all there is (158 -> 154 us for the 256x256 frame; large
+// sorts lose from it, 2,197 -> 2,285 us for 5,000 characters).  Elements handed
+// on by stores to the other CTAs' shared memory instead: 165 us.
+constexpr int kClusterThreads = 512, kClusterWarps = kClusterThreads / 32;
+constexpr int kClusterItems = kRadixTile / kClusterThreads, kClusterWarpTile = 32 * kClusterItems;
 
 // Digit width of pass p of `passes` over `bits` bits, from bit `shift` on.
 __host__ __device__ inline int radix_width(int bits, int shift, int passes, int p) {
@@ -389,11 +395,11 @@ __host__ __device__ inline int radix_width(int bits, int shift, int passes, int 
 }
 
 template <typename K>
-__global__ void __launch_bounds__(kRadixThreads) k_radix_cluster(K *k0, uint32_t *v0, K *k1, uint32_t *v1, uint32_t n,
+__global__ void __launch_bounds__(kClusterThreads) k_radix_cluster(K *k0, uint32_t *v0, K *k1, uint32_t *v1, uint32_t n,
                                                                  int bits, int passes, bool iota,
                                                                  const uint32_t *__restrict__ gsrc,
                                                                  uint32_t *__restrict__ gdst) {
-    __shared__ uint32_t wcnt[kRadixWarps][kRadixDigits];  // running counts, then warp offsets
+    __shared__ uint32_t wcnt[kClusterWarps][kRadixDigits];  // running counts, then warp offsets
     __shared__ uint32_t dcnt[kRadixDigits];               // this block's digit counts, read by the cluster
     __shared__ uint32_t dstart[kRadixDigits], gbase[kRadixDigits];
     __shared__ uint32_t total;
@@ -404,8 +410,8 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_cluster(K *k0, uint32_t
     const int rank = (int)cluster.block_rank(), blocks = (int)cluster.num_blocks();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t lt = (1u << lane) - 1u;
-    const uint32_t blk0 = (uint32_t)rank * kRadixTile, base = blk0 + warp * kRadixWarpTile;
-    constexpr int kPer = kRadixDigits / kRadixThreads;  // digits per thread
+    const uint32_t blk0 = (uint32_t)rank * kRadixTile, base = blk0 + warp * kClusterWarpTile;
+    constexpr int kPer = kRadixDigits / kClusterThreads;  // digits per thread
     for (int p = 0, shift = 0; p < passes; ++p) {
         const int width = radix_width(bits, shift, passes, p);
         const uint32_t mask = (1u << width) - 1u;
@@ -413,20 +419,20 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_cluster(K *k0, uint32_t
         const uint32_t *vi = p & 1 ? v1 : v0;
         K *ko = p & 1 ? k0 : k1;
         uint32_t *vo = p & 1 ? v0 : v1;
-        for (int d = threadIdx.x; d < kRadixWarps * kRadixDigits; d += kRadixThreads) (&wcnt[0][0])[d] = 0;
-        K k[kRadixItems];
-        uint32_t v[kRadixItems], dr[kRadixItems];
+        for (int d = threadIdx.x; d < kClusterWarps * kRadixDigits; d += kClusterThreads) (&wcnt[0][0])[d] = 0;
+        K k[kClusterItems];
+        uint32_t v[kClusterItems], dr[kClusterItems];
 #pragma unroll
-        for (int r = 0; r < kRadixItems; ++r) {
+        for (int r = 0; r < kClusterItems; ++r) {
             // past L1: another CTA of the cluster wrote them in the pass before
             const uint32_t i = base + r * 32 + lane;
             k[r] = i < n ? __ldcg(ki + i) : (K)0;
             v[r] = i >= n ? 0u : (p == 0 && iota ? i : __ldcg(vi + i));
         }
         __syncthreads();
-        // stable rank within the warp's 512 elements, as k_radix_scatter
+        // stable rank within the warp's elements, as k_radix_scatter
 #pragma unroll
-        for (int r = 0; r < kRadixItems; ++r) {
+        for (int r = 0; r < kClusterItems; ++r) {
             const bool ok = base + r * 32 + lane < n;
             const uint32_t d = ok ? (uint32_t)(k[r] >> shift) & mask : (uint32_t)kRadixDigits;
             unsigned peers = __ballot_sync(0xffffffffu, ok);
@@ -447,7 +453,7 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_cluster(K *k0, uint32_t
             const int d = threadIdx.x * kPer + j;
             uint32_t run = 0;
 #pragma unroll
-            for (int w = 0; w < kRadixWarps; ++w) {
+            for (int w = 0; w < kClusterWarps; ++w) {
                 const uint32_t c = wcnt[w][d];
                 wcnt[w][d] = run;
                 run += c;
@@ -481,7 +487,7 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_cluster(K *k0, uint32_t
         }
         __syncthreads();
 #pragma unroll
-        for (int r = 0; r < kRadixItems; ++r) {
+        for (int r = 0; r < kClusterItems; ++r) {
             const uint32_t d = dr[r] & 0xFFFFu;
             if (d < (uint32_t)kRadixDigits) {
                 const uint32_t lp = dstart[d] + wcnt[warp][d] + (dr[r] >> 16);
@@ -492,7 +498,7 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_cluster(K *k0, uint32_t
         __syncthreads();
         const uint32_t cnt = n > blk0 ? min((uint32_t)kRadixTile, n - blk0) : 0u;
         const bool last = p == passes - 1;
-        for (uint32_t q = threadIdx.x; q < cnt; q += kRadixThreads) {
+        for (uint32_t q = threadIdx.x; q < cnt; q += kClusterThreads) {
             const K key = skey[q];
             const uint32_t d = (uint32_t)(key >> shift) & mask;
             const uint32_t g = gbase[d] + (q - dstart[d]);
@@ -524,7 +530,7 @@ static int radix_cluster(K *k0, uint32_t *v0, K *k1, uint32_t *v1, uint32_t n, u
     attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = nb;
-    cfg.blockDim = kRadixThreads;
+    cfg.blockDim = kClusterThreads;
     cfg.dynamicSmemBytes = kDyn;
     cfg.stream = st;
     cfg.attrs = &attr;
