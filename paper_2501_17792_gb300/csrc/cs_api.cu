@@ -969,7 +969,8 @@ static int render_impl(cs_ctx *ctx, const cs_camera *cam, float4 *out, cs_frame_
     if (timing) CS_CUDA(cudaEventRecord(ev[4], st));
     // 5. pair offsets in depth order and pair emission
     // (the per-block sums of the pair counts live in pair_off)
-    launched += bin_scan_sums(ctx->bins_sorted.p, (uint32_t)S, ctx->pair_off.p, ctx->h_pairs, ++ctx->seq, st);
+    launched += bin_scan_sums(ctx->bins_sorted.p, (uint32_t)S, ctx->pair_off.p,
+                              reinterpret_cast<uint32_t *>(ctx->cull.p) + kPairTicketAt, ctx->h_pairs, ++ctx->seq, st);
     CS_CUDA(cudaGetLastError());
     if (stats && S > 0) launched += launch_count_live((uint32_t)S, sorted_keys, ctx->d_meta + kMetaWords - 1, st);
     if (S > 0) CS_TRY(wait_counts(ctx, ctx->h_pairs + 2, ctx->seq));

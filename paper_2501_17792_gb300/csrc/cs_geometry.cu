@@ -102,7 +102,7 @@ int launch_fk(int n_inst, int n_tpl, const int32_t *tid, const float *pose, cons
               int max_depth, float *B, int32_t *cull_scratch, cudaStream_t st) {
     if (n_inst <= 0) return 0;
     int blocks = (n_inst + 7) / 8;
-    k_fk<<<blocks, 256, 0, st>>>(n_inst, n_tpl, tid, pose, tpls, max_depth, B, cull_scratch, kMaxGroups + 3);
+    k_fk<<<blocks, 256, 0, st>>>(n_inst, n_tpl, tid, pose, tpls, max_depth, B, cull_scratch, kFrameTotals);
     return 1;
 }
 
@@ -137,7 +137,9 @@ constexpr int kCullThreads = 1024;
 constexpr uint8_t kHidden = 255;
 // frame totals in the cull scratch (zeroed by k_fk): group counts,
 // then the inverted bits of the lowest depth bound, the highest, the ticket
+// (and the ticket of the pair sums, kPairTicketAt)
 constexpr int kCullZloInv = kMaxGroups, kCullZhi = kMaxGroups + 1, kCullTicket = kMaxGroups + 2;
+static_assert(kCullTicket < kPairTicketAt, "the frame's totals");
 
 __global__ void __launch_bounds__(kCullThreads) k_cull_group(
     int n_inst, int n_tpl, const int32_t *__restrict__ tid, const float *__restrict__ root,
@@ -384,7 +386,7 @@ __global__ void __launch_bounds__(kCullThreads) k_cull_group(
     }
 }
 
-size_t cull_scratch_words(size_t n_inst) { return kMaxGroups + 3 + (n_inst + 3) / 4; }
+size_t cull_scratch_words(size_t n_inst) { return kFrameTotals + (n_inst + 3) / 4; }
 
 int launch_cull_group(int n_inst, int n_tpl, const int32_t *tid, const float *root,
                        const TemplateInfo *tpls, const CamParams &cam, const LodParams &lod,
@@ -394,7 +396,7 @@ int launch_cull_group(int n_inst, int n_tpl, const int32_t *tid, const float *ro
     const unsigned blocks = (unsigned)((n_inst + kCullThreads - 1) / kCullThreads);
     k_cull_group<<<blocks > 0 ? blocks : 1u, kCullThreads, 0, st>>>(
         n_inst, n_tpl, tid, root, tpls, cam, lod, do_cull, V, Cloc, vis, groups, meta, host_meta, host_groups, seq, scratch,
-        reinterpret_cast<uint8_t *>(scratch + kMaxGroups + 3));
+        reinterpret_cast<uint8_t *>(scratch + kFrameTotals));
     return 1;
 }
 

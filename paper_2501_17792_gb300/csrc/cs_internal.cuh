@@ -294,6 +294,8 @@ int launch_fk(int n_inst, int n_tpl, const int32_t *tid, const float *pose, cons
               int max_depth, float *B, int32_t *cull_scratch, cudaStream_t st);
 // Cull scratch of n instances (frame totals, then a group byte per
 // instance), in 4-byte words.
+constexpr int kPairTicketAt = kMaxGroups + 3;        // ticket of the pair sums
+constexpr int kFrameTotals = kPairTicketAt + 1;      // words k_fk clears at the start of the scratch
 size_t cull_scratch_words(size_t n_inst);
 // Runs after launch_fk.  The counts and groups also go to host_meta and
 // host_groups (pinned host memory), then seq to host_meta[kMetaSeq].
@@ -344,8 +346,10 @@ int radix_sort_u16(uint16_t *k0, uint32_t *v0, uint16_t *k1, uint32_t *v1, uint3
 // splat's pairs (the scan's down-sweep fused into the emission) and clears
 // the tile ranges and the compositing's plan counters for the kernels after it.
 size_t bin_scan_blocks(size_t n);
-// host (pinned host memory) receives the total and then seq in host[2].
-int bin_scan_sums(const uint32_t *bins, uint32_t n, uint32_t *sums, uint32_t *host, uint32_t seq, cudaStream_t st);
+// host (pinned host memory) receives the total and then seq in host[2];
+// *ticket is zero (the frame's first kernel clears it).
+int bin_scan_sums(const uint32_t *bins, uint32_t n, uint32_t *sums, uint32_t *ticket, uint32_t *host, uint32_t seq,
+                  cudaStream_t st);
 int launch_emit_pairs_scan(uint32_t n_splats, const uint32_t *order, const uint32_t *bins_sorted,
                            const uint32_t *sums, const float4 *rec, int tiles_x, uint32_t n_tiles, uint16_t *ptile,
                            uint32_t *pval, uint2 *ranges, int32_t *blend_meta, cudaStream_t st);

@@ -56,27 +56,28 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const uint32_t *__
     if (threadIdx.x == 0) sums[blockIdx.x] = total;
 }
 
-// One block: exclusive scan of the tile sums in place, total at sums[nb]
-// (and, when set, at host[0] in pinned host memory, then seq at host[2]).
-__global__ void __launch_bounds__(kScanThreads) k_scan_spine(uint32_t *__restrict__ sums, uint32_t nb, uint32_t *host,
-                                                             uint32_t seq) {
-    __shared__ uint32_t total;
+// Exclusive scan of the block sums in place by one block of kThreads threads,
+// total at sums[nb] and, when set, at host[0] in pinned host memory, then seq
+// at host[2] (read past L1: other CTAs may have written them in this launch).
+template <int kThreads>
+__device__ __forceinline__ void scan_sums(uint32_t *sums, uint32_t nb, uint32_t *total, uint32_t *host, uint32_t seq) {
+    constexpr int kPer = kScanTile / kThreads;
     uint32_t carry = 0;
     for (uint32_t base = 0; base < nb; base += kScanTile) {
-        const uint32_t i0 = base + threadIdx.x * kScanItems;
-        uint32_t v[kScanItems], sum = 0;
+        const uint32_t i0 = base + threadIdx.x * kPer;
+        uint32_t v[kPer], sum = 0;
 #pragma unroll
-        for (int k = 0; k < kScanItems; ++k) {
-            v[k] = i0 + k < nb ? sums[i0 + k] : 0u;
+        for (int k = 0; k < kPer; ++k) {
+            v[k] = i0 + k < nb ? __ldcg(sums + i0 + k) : 0u;
             sum += v[k];
         }
-        uint32_t ex = block_excl_scan(sum, &total) + carry;
+        uint32_t ex = block_excl_scan(sum, total) + carry;
 #pragma unroll
-        for (int k = 0; k < kScanItems; ++k) {
+        for (int k = 0; k < kPer; ++k) {
             if (i0 + k < nb) sums[i0 + k] = ex;
             ex += v[k];
         }
-        carry += total;
+        carry += *total;
     }
     if (threadIdx.x == 0) {
         sums[nb] = carry;
@@ -86,6 +87,11 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_spine(uint32_t *__restric
             *reinterpret_cast<volatile uint32_t *>(host + 2) = seq;
         }
     }
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_scan_spine(uint32_t *sums, uint32_t nb, uint32_t *host, uint32_t seq) {
+    __shared__ uint32_t total;
+    scan_sums<kScanThreads>(sums, nb, &total, host, seq);
 }
 
 template <int MODE>
@@ -696,25 +702,38 @@ __global__ void __launch_bounds__(256) k_emit_pairs(uint32_t n, const uint32_t *
 constexpr int kEmitThreads = 256;
 constexpr int kEmitWarps = kEmitThreads / 32;
 // Blocks of 4,096 splats leave SMs idle below a few million splats (202,738
-// splats are 50 blocks: 21 us, 13 with blocks of 1,024); above, the smaller
-// blocks would only lengthen the one-block scan of the sums.
-constexpr int kEmitRounds = 16, kEmitFewRounds = 4;
-constexpr size_t kEmitFewSplats = (size_t)1 << 22;
+// splats are 50 blocks: 21 us, 13 with blocks of 1,024, 8 with
+// blocks of 256); larger frames would only lengthen the one-block scan of the
+// sums with smaller blocks.
+constexpr int kEmitRounds = 16, kEmitFewRounds = 4, kEmitOneRound = 1;
+constexpr size_t kEmitFewSplats = (size_t)1 << 22, kEmitOneSplats = (size_t)1 << 18;
 
+// Pair counts of the blocks.  With the smallest blocks (few splats) the CTA
+// that finishes last (a ticket taken after a memory fence) scans them, which
+// as a launch of its own costs such a frame 4 us (16,384 splats 153 -> 148 us,
+// 202,738 splats 334 -> 328 us a frame with the smaller blocks); with
+// thousands of CTAs the fences cost more than the launch (22.7 M splats 2,664
+// -> 2,680 us).
 template <int kRounds>
 __global__ void __launch_bounds__(kEmitThreads) k_bin_sums(const uint32_t *__restrict__ bins, uint32_t n,
-                                                           uint32_t *__restrict__ sums) {
-    __shared__ uint32_t wsum[kEmitWarps];
+                                                           uint32_t *sums, uint32_t *ticket, uint32_t *host,
+                                                           uint32_t seq) {
+    __shared__ uint32_t wsum[kEmitWarps], total;
+    __shared__ bool last;
     const uint32_t base = blockIdx.x * (kEmitThreads * kRounds);
     uint32_t v = 0;
+    if (kRounds == 1) {
+        if (base + threadIdx.x < n) v = bin_count(bins[base + threadIdx.x]);
+    } else {
 #pragma unroll
-    for (int j = 0; j < kRounds / 4; ++j) {
-        const uint32_t i = base + (j * kEmitThreads + threadIdx.x) * 4u;
-        if (i + 4u <= n) {
-            const uint4 w = __ldg(reinterpret_cast<const uint4 *>(bins + i));  // (the words start 16-byte aligned)
-            v += bin_count(w.x) + bin_count(w.y) + bin_count(w.z) + bin_count(w.w);
-        } else {
-            for (uint32_t k = i; k < n; ++k) v += bin_count(bins[k]);
+        for (int j = 0; j < kRounds / 4; ++j) {
+            const uint32_t i = base + (j * kEmitThreads + threadIdx.x) * 4u;
+            if (i + 4u <= n) {
+                const uint4 w = __ldg(reinterpret_cast<const uint4 *>(bins + i));  // (the words start 16-byte aligned)
+                v += bin_count(w.x) + bin_count(w.y) + bin_count(w.z) + bin_count(w.w);
+            } else {
+                for (uint32_t k = i; k < n; ++k) v += bin_count(bins[k]);
+            }
         }
     }
     v = __reduce_add_sync(0xffffffffu, v);
@@ -724,6 +743,16 @@ __global__ void __launch_bounds__(kEmitThreads) k_bin_sums(const uint32_t *__res
         uint32_t t = 0;
         for (int w = 0; w < kEmitWarps; ++w) t += wsum[w];
         sums[blockIdx.x] = t;
+        if (kRounds == kEmitOneRound) {
+            __threadfence();
+            last = atomicAdd(ticket, 1u) == gridDim.x - 1u;
+        }
+    }
+    if (kRounds == kEmitOneRound) {
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+        scan_sums<kEmitThreads>(sums, gridDim.x, &total, host, seq);
     }
 }
 
@@ -821,16 +850,25 @@ __global__ void __launch_bounds__(kEmitThreads, 8)
     }
 }
 
-// splats of a block of the two kernels above
-static uint32_t emit_tile(size_t n) { return kEmitThreads * (n <= kEmitFewSplats ? kEmitFewRounds : kEmitRounds); }
+// rounds of a block of the two kernels above
+static int emit_rounds(size_t n) {
+    return n <= kEmitOneSplats ? kEmitOneRound : n <= kEmitFewSplats ? kEmitFewRounds : kEmitRounds;
+}
 
-size_t bin_scan_blocks(size_t n) { return (n + emit_tile(n) - 1) / emit_tile(n); }
+size_t bin_scan_blocks(size_t n) {
+    const size_t tile = (size_t)kEmitThreads * emit_rounds(n);
+    return (n + tile - 1) / tile;
+}
 
-int bin_scan_sums(const uint32_t *bins, uint32_t n, uint32_t *sums, uint32_t *host, uint32_t seq, cudaStream_t st) {
+int bin_scan_sums(const uint32_t *bins, uint32_t n, uint32_t *sums, uint32_t *ticket, uint32_t *host, uint32_t seq,
+                  cudaStream_t st) {
     if (n == 0) return 0;
     const uint32_t nb = (uint32_t)bin_scan_blocks(n);
-    if (n <= kEmitFewSplats) k_bin_sums<kEmitFewRounds><<<nb, kEmitThreads, 0, st>>>(bins, n, sums);
-    else k_bin_sums<kEmitRounds><<<nb, kEmitThreads, 0, st>>>(bins, n, sums);
+    switch (emit_rounds(n)) {
+        case kEmitOneRound: k_bin_sums<kEmitOneRound><<<nb, kEmitThreads, 0, st>>>(bins, n, sums, ticket, host, seq); return 1;
+        case kEmitFewRounds: k_bin_sums<kEmitFewRounds><<<nb, kEmitThreads, 0, st>>>(bins, n, sums, nullptr, nullptr, 0u); break;
+        default: k_bin_sums<kEmitRounds><<<nb, kEmitThreads, 0, st>>>(bins, n, sums, nullptr, nullptr, 0u); break;
+    }
     k_scan_spine<<<1, kScanThreads, 0, st>>>(sums, nb, host, seq);
     return 2;
 }
@@ -840,12 +878,20 @@ int launch_emit_pairs_scan(uint32_t n_splats, const uint32_t *order, const uint3
                            uint32_t *pval, uint2 *ranges, int32_t *blend_meta, cudaStream_t st) {
     if (n_splats == 0) return 0;
     const uint32_t nb = (uint32_t)bin_scan_blocks(n_splats);
-    if (n_splats <= kEmitFewSplats)
-        k_emit_pairs_scan<kEmitFewRounds><<<nb, kEmitThreads, 0, st>>>(n_splats, order, bins_sorted, sums, rec, tiles_x,
-                                                                      n_tiles, ptile, pval, ranges, blend_meta);
-    else
-        k_emit_pairs_scan<kEmitRounds><<<nb, kEmitThreads, 0, st>>>(n_splats, order, bins_sorted, sums, rec, tiles_x,
-                                                                   n_tiles, ptile, pval, ranges, blend_meta);
+    switch (emit_rounds(n_splats)) {
+        case kEmitOneRound:
+            k_emit_pairs_scan<kEmitOneRound><<<nb, kEmitThreads, 0, st>>>(n_splats, order, bins_sorted, sums, rec, tiles_x,
+                                                                         n_tiles, ptile, pval, ranges, blend_meta);
+            break;
+        case kEmitFewRounds:
+            k_emit_pairs_scan<kEmitFewRounds><<<nb, kEmitThreads, 0, st>>>(n_splats, order, bins_sorted, sums, rec, tiles_x,
+                                                                          n_tiles, ptile, pval, ranges, blend_meta);
+            break;
+        default:
+            k_emit_pairs_scan<kEmitRounds><<<nb, kEmitThreads, 0, st>>>(n_splats, order, bins_sorted, sums, rec, tiles_x,
+                                                                       n_tiles, ptile, pval, ranges, blend_meta);
+            break;
+    }
     return 1;
 }
 
