@@ -88,7 +88,8 @@ int cs_lod_rank(cs_ctx *ctx, const float *score, uint32_t *order_out);
 
 /* ---------------------------------------------------------------------
  * The ranking MLP: 48 -> 64 -> 64 -> 1, ReLU, hand-written BF16 tensor-core
- * kernels (mma m16n8k16, FP32 accumulate).  Rounding points (the FP64
+ * kernels (mma.sync in the forward pass, tcgen05 in training; FP32
+ * accumulate).  Rounding points (the FP64
  * reference rounds at the same places): inputs, W1, W2, the first hidden
  * activations and the back-propagated pre-activation gradients are BF16;
  * biases, w3, the second hidden layer, the output and all sums are FP32.
@@ -120,7 +121,9 @@ int cs_mlp_forward(cs_mlp *m, int64_t n, const float *feat, const int32_t *band,
  * [n]) with loss (1/n) sum (y - target)^2 and learning rate lr > 0.
  * *loss_out (HOST, may be NULL) receives the batch loss before the step
  * (the call then synchronises the stream).  Errors: CS_ERR_ARG (n < 1,
- * lr <= 0, NULL or misaligned arrays), CS_ERR_OOM, CS_ERR_CUDA. */
+ * lr <= 0, NULL or misaligned arrays), CS_ERR_OOM, CS_ERR_CUDA (also when
+ * the training kernel gave up waiting for its products: the parameters then
+ * keep their values until cs_mlp_set_params). */
 int cs_mlp_train_step(cs_mlp *m, int64_t n, const float *feat, const int32_t *band, const float *target,
                       float lr, float *loss_out);
 

@@ -21,7 +21,8 @@ def _pairs_of(rec, live_order, tiles_x):
 
 
 @pytest.mark.parametrize("n,instances,size", [(1, 1, 0.3), (33, 1, 0.05), (1024, 1, 0.3), (1025, 1, 0.01), (4099, 2, 0.02),
-                                              (9000, 3, 0.002), (66000, 64, 0.001)])
+                                              (9000, 3, 0.002), (9000, 40, 0.002),
+                                              (66000, 64, 0.001)])
 def test_pairs_of_the_reach_boxes(n, instances, size):
     from paper_2501_17792_gb300 import binding
     from tests import scene_util as U
