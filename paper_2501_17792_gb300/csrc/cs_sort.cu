@@ -688,17 +688,18 @@ __global__ void __launch_bounds__(256) k_emit_pairs(uint32_t n, const uint32_t *
 // takes 256 kRounds splats in depth order, warp w the 32 kRounds from
 // w 32 kRounds on; the warp's offset is the scanned block sum plus the
 // totals of the warps before it, so there is one barrier and no per-splat
-// offset array.  Each round of 32 splats is scanned in the warp and its
+// offset array.  Each step of 64 splats, two a lane, is scanned in the warp and its
 // pairs are written 32 at a time, one per lane: the lanes whose splats have
 // pairs leave them compacted in shared memory, a bit per splat start in the
 // window of 32 pairs (one reduction) tells each lane its splat, and the pair's rank among the
 // splat's tiles its tile (row-major; a 3x3 mask by a table of the positions
 // of its set bits).  Exactly the pairs emit_splat_pairs writes, in their
 // order.
-// Bound by instruction issue (about 150 per 32 splats and their pairs).
-// 42.5 M pairs of 22.7 M splats: 228 -> 178 us against 1,024-thread blocks
-// with three barriers a round, small splats written by their own threads and
-// larger ones queued; the sums before it 27 -> 18 us (16-byte loads).
+// Bound by instruction issue (about 400 per 64 splats and their 90 pairs).
+// 42.5 M pairs of 22.7 M splats: 228 us with 1,024-thread blocks, three
+// barriers a round, small splats written by their own threads and larger ones
+// queued; 178 with warps of 32 splats a step; 162 with 64 (fewer scans and
+// fuller windows).  The sums before it 27 -> 18 us (16-byte loads).
 constexpr int kEmitThreads = 256;
 constexpr int kEmitWarps = kEmitThreads / 32;
 // Blocks of 4,096 splats leave SMs idle below a few million splats (202,738
@@ -756,13 +757,34 @@ __global__ void __launch_bounds__(kEmitThreads) k_bin_sums(const uint32_t *__res
     }
 }
 
+// Words i and i + 1 (i even, the array 8-byte aligned); zero from `end` on.
+__device__ __forceinline__ uint2 load_two(const uint32_t *__restrict__ p, uint32_t i, uint32_t end) {
+    if (i + 1u < end) return __ldg(reinterpret_cast<const uint2 *>(p + i));
+    return make_uint2(i < end ? p[i] : 0u, 0u);
+}
+
+// A splat with pairs as its warp's lanes read it: splat id, first pair, tile
+// x0 | y0 << 16, mask or kBinLarge | tiles per row.
+__device__ __forceinline__ uint4 staged_splat(uint32_t b, uint32_t s, uint32_t first, const float4 *__restrict__ rec,
+                                              uint32_t n) {
+    uint4 e = make_uint4(s, first, (b & 0xFFu) | ((b & 0xFF00u) << 8), (b >> 16) & 0x1FFu);
+    if ((b & kBinLarge) && in_bounds(s < n, kChkSplat)) {
+        const float4 q = rec[(size_t)s * kRecVec];  // reach x, reach y, log2 o, C
+        const uint32_t rx = __float_as_uint(q.x), ry = __float_as_uint(q.y);
+        const uint32_t x0 = (rx & 0xFFFFu) >> 4, y0 = (ry & 0xFFFFu) >> 4;
+        e.z = x0 | (y0 << 16);
+        e.w = kBinLarge | (((rx >> 16) >> 4) - x0 + 1u);
+    }
+    return e;
+}
+
 template <int kRounds>
 __global__ void __launch_bounds__(kEmitThreads, 8)
     k_emit_pairs_scan(uint32_t n, const uint32_t *__restrict__ order, const uint32_t *__restrict__ bins,
                       const uint32_t *__restrict__ sums, const float4 *__restrict__ rec, int tiles_x,
                       uint32_t n_tiles, uint16_t *__restrict__ ptile, uint32_t *__restrict__ pval,
                       uint2 *__restrict__ ranges, int32_t *__restrict__ blend_meta) {
-    __shared__ uint4 stage[kEmitWarps][32];  // splat id, first pair, tile x0 | y0 << 16, mask or large | tiles per row
+    __shared__ uint4 stage[kEmitWarps][64];
     __shared__ uint32_t nth[512];            // positions of a mask's first eight set bits, four bits each
     __shared__ uint32_t wsum[kEmitWarps];
     for (uint32_t k = blockIdx.x * kEmitThreads + threadIdx.x; k < n_tiles; k += gridDim.x * kEmitThreads)
@@ -781,42 +803,39 @@ __global__ void __launch_bounds__(kEmitThreads, 8)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t lt = (1u << lane) - 1u;
     const uint32_t base = (blockIdx.x * kEmitWarps + warp) * (32u * kRounds);
-    uint32_t mine = 0;
+    const uint32_t end = min(n, base + 32u * kRounds);
+    constexpr int kSteps = (kRounds + 1) / 2;  // of 64 splats, two consecutive ones a lane
+    uint32_t i = base + 2 * lane, mine = 0;
 #pragma unroll
-    for (int r = 0; r < kRounds; ++r) mine += base + r * 32 + lane < n ? bin_count(bins[base + r * 32 + lane]) : 0u;
+    for (int r = 0; r < kSteps; ++r) {
+        const uint2 b = load_two(bins, i + 64 * r, end);
+        mine += bin_count(b.x) + bin_count(b.y);
+    }
     mine = __reduce_add_sync(0xffffffffu, mine);
     if (lane == 0) wsum[warp] = mine;
     __syncthreads();
     if (mine == 0u) return;
     uint32_t o0 = sums[blockIdx.x];
     for (int w = 0; w < warp; ++w) o0 += wsum[w];
-    // bin words are read two rounds ahead, splat ids one
-    uint32_t i = base + lane;
-    uint32_t b = i < n ? bins[i] : 0u, b1 = i + 32u < n ? bins[i + 32] : 0u;
-    uint32_t s = bin_count(b) ? order[i] : 0u;
+    // bin words are read two steps ahead, splat ids one
+    uint2 b = load_two(bins, i, end), b1 = load_two(bins, i + 64u, end);
+    uint2 s = bin_count(b.x) + bin_count(b.y) ? load_two(order, i, end) : make_uint2(0u, 0u);
 #pragma unroll 1
-    for (int r = 0; r < kRounds; ++r, i += 32) {
-        const uint32_t b2 = r + 2 < kRounds && i + 64u < n ? bins[i + 64] : 0u;
-        const uint32_t s1 = r + 1 < kRounds && bin_count(b1) ? order[i + 32] : 0u;
-        const uint32_t c = bin_count(b);
-        const uint32_t incl = warp_inclusive_scan(c), first = incl - c;
+    for (int r = 0; r < kSteps; ++r, i += 64) {
+        const uint2 b2 = load_two(bins, i + 128u, end);
+        const uint2 s1 = bin_count(b1.x) + bin_count(b1.y) ? load_two(order, i + 64u, end) : make_uint2(0u, 0u);
+        const uint32_t c0 = bin_count(b.x), c1 = bin_count(b.y);
+        const uint32_t incl = warp_inclusive_scan(c0 + c1), first0 = incl - c0 - c1, first1 = incl - c1;
         const uint32_t pairs = __shfl_sync(0xffffffffu, incl, 31);
-        const unsigned have = __ballot_sync(0xffffffffu, c != 0u);
-        if (c) {
-            uint4 e = make_uint4(s, first, (b & 0xFFu) | ((b & 0xFF00u) << 8), (b >> 16) & 0x1FFu);
-            if ((b & kBinLarge) && in_bounds(s < n, kChkSplat)) {
-                const float4 q = rec[(size_t)s * kRecVec];  // reach x, reach y, log2 o, C
-                const uint32_t rx = __float_as_uint(q.x), ry = __float_as_uint(q.y);
-                const uint32_t x0 = (rx & 0xFFFFu) >> 4, y0 = (ry & 0xFFFFu) >> 4;
-                e.z = x0 | (y0 << 16);
-                e.w = kBinLarge | (((rx >> 16) >> 4) - x0 + 1u);
-            }
-            stage[warp][__popc(have & lt)] = e;
-        }
+        const unsigned have0 = __ballot_sync(0xffffffffu, c0 != 0u), have1 = __ballot_sync(0xffffffffu, c1 != 0u);
+        const uint32_t at = __popc(have0 & lt) + __popc(have1 & lt);
+        if (c0) stage[warp][at] = staged_splat(b.x, s.x, first0, rec, n);
+        if (c1) stage[warp][at + (c0 != 0u)] = staged_splat(b.y, s.y, first1, rec, n);
         __syncwarp();
         uint32_t started = 0;
         for (uint32_t w0 = 0; w0 < pairs; w0 += 32u) {
-            const unsigned starts = __reduce_or_sync(0xffffffffu, c && first - w0 < 32u ? 1u << (first - w0) : 0u);
+            const unsigned starts = __reduce_or_sync(0xffffffffu, (c0 && first0 - w0 < 32u ? 1u << (first0 - w0) : 0u) |
+                                                                      (c1 && first1 - w0 < 32u ? 1u << (first1 - w0) : 0u));
             const uint32_t p = w0 + lane;
             const uint32_t owner = started + __popc(starts & (lt | (1u << lane))) - 1u;
             started += __popc(starts);
@@ -826,9 +845,10 @@ __global__ void __launch_bounds__(kEmitThreads, 8)
             uint32_t row, col;
             if (e.w & kBinLarge) {
                 // k / width: exact for k < 2^16 (the quotient is at least half
-                // a width's inverse away from an integer)
+                // a width's inverse away from an integer, the reciprocal's
+                // error a few ulp)
                 const uint32_t width = e.w & ~kBinLarge;
-                row = (uint32_t)(((float)k + 0.5f) * (1.0f / (float)width));
+                row = (uint32_t)(((float)k + 0.5f) * __fdividef(1.0f, (float)width));
                 col = k - row * width;
             } else {
                 const uint32_t at = k < 8u ? (nth[e.w] >> (4u * k)) & 15u : 8u;
