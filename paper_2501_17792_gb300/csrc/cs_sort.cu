@@ -688,13 +688,13 @@ __global__ void __launch_bounds__(256) k_emit_pairs(uint32_t n, const uint32_t *
 // takes 256 kRounds splats in depth order, warp w the 32 kRounds from
 // w 32 kRounds on; the warp's offset is the scanned block sum plus the
 // totals of the warps before it, so there is one barrier and no per-splat
-// offset array.  Each step of 64 splats, two a lane, is scanned in the warp and its
-// pairs are written 32 at a time, one per lane: the lanes whose splats have
-// pairs leave them compacted in shared memory, a bit per splat start in the
-// window of 32 pairs (one reduction) tells each lane its splat, and the pair's rank among the
-// splat's tiles its tile (row-major; a 3x3 mask by a table of the positions
-// of its set bits).  Exactly the pairs emit_splat_pairs writes, in their
-// order.
+// offset array.  Each step of 64 splats, two a lane, is scanned in the warp
+// and its pairs are written 32 at a time, one per lane: the splats with pairs
+// are left compacted in shared memory, a bit per splat start in the window of
+// 32 pairs (one reduction) tells each lane its splat, and the pair's rank
+// among the splat's tiles its tile (row-major; a 3x3 mask by a table of the
+// positions of its set bits).  Exactly the pairs emit_splat_pairs writes, in
+// their order.
 // Bound by instruction issue (about 400 per 64 splats and their 90 pairs).
 // 42.5 M pairs of 22.7 M splats: 228 us with 1,024-thread blocks, three
 // barriers a round, small splats written by their own threads and larger ones
