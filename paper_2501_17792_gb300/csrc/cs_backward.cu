@@ -88,8 +88,10 @@ struct BwdWarp {
     float rows[kBwdRows][kBwdLd];
 };
 
-// Adds the sums of the first n rows to dsplat, lane l row l at float dst.
-__device__ __forceinline__ void flush_rows(const BwdWarp &sh, int n, uint32_t dst, float *__restrict__ dsplat) {
+// Adds the sums of the first n rows to dsplat; row l, taken by lane l, is sum
+// l % kBwdGrads of the splat the lane names.  (The address needs 64 bits: a
+// frame may hold more than 2^32 / 12 splats.)
+__device__ __forceinline__ void flush_rows(const BwdWarp &sh, int n, uint32_t splat, float *__restrict__ dsplat) {
     const int lane = threadIdx.x & 31;
     __syncwarp();
     if (lane < n) {
@@ -104,7 +106,7 @@ __device__ __forceinline__ void flush_rows(const BwdWarp &sh, int n, uint32_t ds
             t.w += v.w;
         }
         const float x = (t.x + t.y) + (t.z + t.w);
-        if (x != 0.0f) atomicAdd(dsplat + dst, x);
+        if (x != 0.0f) atomicAdd(dsplat + (size_t)splat * 12u + lane % kBwdGrads, x);
     }
     __syncwarp();
 }
@@ -170,7 +172,7 @@ __global__ void __launch_bounds__(kBwdThreads, 5) k_blend_backward(
     }
     const uint32_t top = __reduce_max_sync(0xffffffffu, end);
     int n_rows = 0;
-    uint32_t dst = 0u;
+    uint32_t splat = 0u;  // of the lane's row
     uint32_t base = lo + ((top - 1u - lo) & ~31u);
     uint32_t i = base + (uint32_t)lane;
     if (top <= lo) return;
@@ -229,11 +231,10 @@ __global__ void __launch_bounds__(kBwdThreads, 5) k_blend_backward(
             const float v[kBwdGrads] = {G, Gx, Gy, Gx * dx, Gx * dy, Gy * dy, gr, gg, gb};
 #pragma unroll
             for (int e = 0; e < kBwdGrads; ++e) sh.rows[n_rows + e][lane] = v[e];
-            const uint32_t e = (uint32_t)(lane - n_rows);
-            if (e < (uint32_t)kBwdGrads) dst = __float_as_uint(b.w) * 12u + e;
+            if ((uint32_t)(lane - n_rows) < (uint32_t)kBwdGrads) splat = __float_as_uint(b.w);
             n_rows += kBwdGrads;
             if (n_rows == kBwdRows) {
-                flush_rows(sh, kBwdRows, dst, dsplat);
+                flush_rows(sh, kBwdRows, splat, dsplat);
                 n_rows = 0;
             }
         }
@@ -243,7 +244,7 @@ __global__ void __launch_bounds__(kBwdThreads, 5) k_blend_backward(
         i -= 32u;
         s = s_next;
     }
-    flush_rows(sh, n_rows, dst, dsplat);
+    flush_rows(sh, n_rows, splat, dsplat);
 }
 
 // ---------------------------------------------------------------------------

@@ -1,0 +1,53 @@
+"""Gradients at the limits of their index range: frames of more than 2^32 / 12
+splats."""
+import numpy as np
+import pytest
+
+from tests import scene_util as U
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _renderer(sc, **kw):
+    from paper_2501_17792_gb300 import binding
+    r = binding.Renderer(device=0, **kw)
+    r.upload_templates(sc.templates)
+    r.set_instances(sc.instances.template_id, sc.instances.root, sc.instances.pose)
+    return r
+
+
+def test_gradients_of_splats_past_two_to_the_32_sums():
+    """Twelve floats of sums a splat: from splat 2^32 / 12 on their address
+    needs more than 32 bits.  A frame of 357.9 million splats, all behind the
+    camera but the last two instances', has the gradients of a frame of those
+    two."""
+    n, seen = 4096, 2
+    hidden = 2 ** 32 // 12 // n + 2
+    # 120 bytes a splat and a quarter more, and what the caller holds
+    if torch.cuda.mem_get_info()[0] < 70 << 30:
+        pytest.skip("needs 70 GB of device memory")
+    rng = np.random.default_rng(5)
+    tpl = U.template_from(rng.uniform(-0.3, 0.3, (n, 3)), rng.uniform(0.01, 0.03, (n, 3)), rng.standard_normal((n, 4)),
+                          rng.uniform(0.1, 0.9, n), 0.3 * rng.standard_normal((n, 1, 3)))
+    front = np.tile(np.eye(3, 4, dtype=np.float32), (seen, 1, 1))
+    front[:, :, 3] = [[-0.3, 0.0, 2.5], [0.3, 0.1, 2.6]]
+    back = np.tile(np.eye(3, 4, dtype=np.float32), (hidden, 1, 1))
+    back[:, 2, 3] = -5.0
+    cam = U.identity_camera(64, 48, 60.0)
+    dl = torch.randn((48, 64, 4), generator=torch.Generator(device="cuda").manual_seed(2), device="cuda")
+    got = []
+    for roots in (front, np.concatenate([back, front])):
+        r = _renderer(U.scene_of([tpl], U.instances(len(roots), roots), cam), instance_cull=False)
+        img, st = r.render_train(cam, stats=True)
+        assert st["splats"] == len(roots) * n
+        g = r.backward(dl, len(roots))
+        torch.cuda.synchronize()
+        g["pose"] = g["pose"][-seen:].clone()
+        got.append(dict(g, img=img))
+        r.close()
+    assert torch.equal(got[0]["img"], got[1]["img"])
+    for k, a in got[0].items():
+        # the sums reach a value in any order
+        assert float(a.abs().max()) > 0.0
+        assert torch.allclose(got[1][k], a, rtol=1e-4, atol=1e-5 * float(a.abs().max())), k
