@@ -167,11 +167,17 @@ __device__ __forceinline__ float splat_alpha(float dx, float dy, float a, float 
     return keep_alpha(dx, dy, radius, p, __fadd_rn(p, lo), kAlphaMin);
 }
 
+// The colour of a splat with weight zero must not count: zero times an
+// infinite colour is NaN.  kWild: some of the staged colours are not finite.
+template <bool kWild>
 __device__ __forceinline__ void add_colour(const HitStage &st, int k, Pixel &px, f2 w) {
     const ulonglong2 gb = st.gb[k];
-    px.r = fma2(st.rr[k].y, w, px.r);
-    px.g = fma2(gb.x, w, px.g);
-    px.b = fma2(gb.y, w, px.b);
+    const auto used = [w](f2 c) {
+        return kWild ? pack2(lo2(w) > 0.0f ? lo2(c) : 0.0f, hi2(w) > 0.0f ? hi2(c) : 0.0f) : c;
+    };
+    px.r = fma2(used(st.rr[k].y), w, px.r);
+    px.g = fma2(used(gb.x), w, px.g);
+    px.b = fma2(used(gb.y), w, px.b);
 }
 
 // kMode 0: colour only; 1 (statistics): also add every composited weight
@@ -181,7 +187,7 @@ enum { kPlain = 0, kStats = 1, kTraining = 2 };
 
 // The staged hits composited in order, with the stop rule.  Every lane of
 // the warp calls it.
-template <int kMode>
+template <int kMode, bool kWild>
 __device__ __forceinline__ void walk_hits(const HitStage &st, int cnt, Pixel &px, float *__restrict__ contrib) {
 #pragma unroll 1
     for (int k = 0; 2 * k < cnt; ++k) {
@@ -204,7 +210,7 @@ __device__ __forceinline__ void walk_hits(const HitStage &st, int cnt, Pixel &px
             }
         }
         const float w0 = a0 * px.T, w1 = a1 * T1;
-        add_colour(st, k, px, pack2(w0, w1));
+        add_colour<kWild>(st, k, px, pack2(w0, w1));
         px.T = T2;
         if (kMode == kTraining) {
             if (a0 > 0.0f) px.last = st.id[2 * k];
@@ -228,23 +234,27 @@ __device__ __forceinline__ bool meets_block(const float4 &q, int bx0, int by0) {
            (int)(ry & 0xFFFFu) <= by0 + kBlockH - 1 && (int)(ry >> 16) >= by0;
 }
 
-// Stage the lanes' pairs whose reach box meets the block; returns how many.
+// Stage the lanes' pairs whose reach box meets the block; returns how many,
+// and in `wild` whether a colour among them is not finite (their sum is not).
 // Only those load the other 32 bytes of their record.
 template <int kMode>
 __device__ __forceinline__ int stage_hits(HitStage &st, bool have, uint32_t s, const float4 &q, uint32_t pair,
-                                          const float4 *__restrict__ rec, int bx0, int by0) {
+                                          const float4 *__restrict__ rec, int bx0, int by0, bool &wild) {
     const int lane = threadIdx.x & 31;
     const bool mine = have && meets_block(q, bx0, by0);
     const uint32_t m = __ballot_sync(0xffffffffu, mine);
     const int cnt = __popc(m);
+    bool odd = false;
     if (mine) {
         const float4 *p = rec + (size_t)s * kRecVec;
         const float4 a = __ldg(p + 1), c = __ldg(p + 2);
         const int pos = __popc(m & ((1u << lane) - 1u));
         stage_hit(st, pos, q, a, c);
+        odd = !(c.x + c.y + c.z < INFINITY);
         if (kMode != kPlain) st.id[pos] = kMode == kStats ? s : pair + 1u;
     }
     if (lane == 0 && (cnt & 1)) stage_pad(st, cnt);
+    wild = __any_sync(0xffffffffu, odd);
     return cnt;
 }
 
@@ -349,12 +359,14 @@ __device__ __forceinline__ void warp_walk(HitStage &st, uint32_t start, uint32_t
     for (uint32_t base = start; base < end; base += 32u, i += 32u) {
         if (kMode == kTraining && groups && !closed(px))
             store_boundary(work, start, base, (int)threadIdx.x, pixel_state(px, px.T));
-        const int cnt = stage_hits<kMode>(st, i < end, s, q, i, rec, bx0, by0);
+        bool wild;
+        const int cnt = stage_hits<kMode>(st, i < end, s, q, i, rec, bx0, by0, wild);
         s = s1;
         if (i + 32u < end) q = __ldg(rec + (size_t)s * kRecVec);
         if (i + 64u < end) s1 = __ldg(pval + i + 64);
         __syncwarp();
-        walk_hits<kMode>(st, cnt, px, work.contrib);
+        if (wild) walk_hits<kMode, true>(st, cnt, px, work.contrib);
+        else walk_hits<kMode, false>(st, cnt, px, work.contrib);
         __syncwarp();  // the staging buffer is refilled by the next batch
         const uint32_t next = base + 32u;
         bool settled = true;
