@@ -617,6 +617,7 @@ __global__ void __launch_bounds__(kBwdThreads, 3) k_project_backward(
         float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
         for (int i = slice; i < n; i += kSlices) {
             const float w = sh.W[i][j];
+            if (w == 0.f) continue;  // (most; and a gradient that is not finite stays with its joints)
             const float4 v = sh.M[i][r];
             a.x += w * v.x;
             a.y += w * v.y;

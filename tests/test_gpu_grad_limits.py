@@ -1,5 +1,8 @@
-"""Gradients at the limits of their index range: frames of more than 2^32 / 12
-splats."""
+"""Gradients at the limits of their index ranges and of their values: frames
+of more than 2^32 / 12 splats, and values that are not finite, which spoil
+what they belong to and nothing else."""
+import math
+
 import numpy as np
 import pytest
 
@@ -51,3 +54,37 @@ def test_gradients_of_splats_past_two_to_the_32_sums():
         # the sums reach a value in any order
         assert float(a.abs().max()) > 0.0
         assert torch.allclose(got[1][k], a, rtol=1e-4, atol=1e-5 * float(a.abs().max())), k
+
+
+def _two_gaussians(**kw):
+    """Gaussians skinned to the left and to the right leg alone, in different
+    8x4 pixel blocks of a 32 x 16 view."""
+    z, f = 2.0, 30.0
+    px = np.array([[6.5, 6.5], [25.5, 9.5]])
+    means = np.stack([(px[:, 0] - 16) * z / f, (px[:, 1] - 8) * z / f, np.full(2, z)], 1)
+    tpl = U.template_from(means, [[0.03, 0.05, 0.07], [0.06, 0.04, 0.05]], [[0.8, 0.2, 0.3, -0.1], [0.9, -0.3, 0.2, 0.2]],
+                          np.full(2, 0.5),
+                          **dict(dict(sh=np.full((2, 1, 3), 0.3), skin_idx=[[4, 5, 2, 3], [5, 4, 1, 3]]), **kw))
+    return U.scene_of([tpl], U.instances(1), U.identity_camera(32, 16, f))
+
+
+@pytest.mark.parametrize("bad", [math.nan, math.inf])
+def test_a_bad_pixel_spoils_the_joints_of_its_gaussians_only(bad):
+    sc = _two_gaussians()
+    r = _renderer(sc)
+    out = []
+    for v in (0.0, bad):
+        dl = torch.ones((16, 32, 4), device="cuda")
+        dl[6, 6] = v  # a pixel of the first Gaussian
+        r.render_train(sc.camera)
+        out.append({k: v.cpu().numpy() for k, v in r.backward(dl, 1).items()})
+    r.close()
+    good, bad_ = out
+    # joint 5 hangs from joint 2, joint 4 (the first Gaussian's) from joint 1
+    assert not np.isfinite(bad_["pose"][0, 4]).all()
+    assert np.abs(good["pose"][0, 5]).max() > 0.0
+    # (the pixels' sums reach a value in any order)
+    close = lambda a, b: np.allclose(a, b, rtol=1e-4, atol=1e-5 * np.abs(b).max())
+    assert close(bad_["pose"][0, [2, 5]], good["pose"][0, [2, 5]])
+    for k in ("means", "scales", "quats", "opacity", "sh"):
+        assert close(bad_[k][1], good[k][1]), k
