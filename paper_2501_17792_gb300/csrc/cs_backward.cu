@@ -330,7 +330,8 @@ __device__ __forceinline__ void sh_backward(const float4 *__restrict__ sh, int n
             const int f = 4 * p + q;
             if (f >= 3 * K) continue;
             g[q] = Y[f / 3] * gc[f % 3];
-            const float cf = e[q] * gc[f % 3];
+            // (a channel without gradient adds nothing, whatever its coefficients)
+            const float cf = gc[f % 3] != 0.f ? e[q] * gc[f % 3] : 0.f;
             gd[0] += cf * dY[f / 3][0];
             gd[1] += cf * dY[f / 3][1];
             gd[2] += cf * dY[f / 3][2];

@@ -88,3 +88,23 @@ def test_a_bad_pixel_spoils_the_joints_of_its_gaussians_only(bad):
     assert close(bad_["pose"][0, [2, 5]], good["pose"][0, [2, 5]])
     for k in ("means", "scales", "quats", "opacity", "sh"):
         assert close(bad_[k][1], good[k][1]), k
+
+
+@pytest.mark.parametrize("coefficient", [-math.inf, math.nan])
+def test_a_channel_clamped_at_zero_passes_no_gradient_whatever_its_coefficients(coefficient):
+    """The red channel is clamped for any very negative coefficient: the same
+    gradients as for -100."""
+    out = []
+    for v in (-100.0, coefficient):
+        sh = 0.2 * np.random.default_rng(3).standard_normal((2, 4, 3))
+        sh[0, 0, 0] = v
+        sc = _two_gaussians(sh=sh)
+        r = _renderer(sc)
+        img = r.render_train(sc.camera).cpu().numpy()
+        assert img[6, 6, 0] == 0.0 and img[6, 6, 1] > 0.0
+        dl = torch.ones((16, 32, 4), device="cuda")
+        out.append({k: g.cpu().numpy() for k, g in r.backward(dl, 1).items()})
+        r.close()
+    for k, a in out[0].items():
+        assert np.abs(a).max() > 0.0
+        assert np.allclose(out[1][k], a, rtol=1e-4, atol=1e-5 * np.abs(a).max()), k
