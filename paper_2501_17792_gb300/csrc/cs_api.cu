@@ -1,6 +1,7 @@
 // cs_api.cu -- the C ABI of libcrowdsplat.so (declared in include/crowdsplat.h):
 // context and device-memory management, template upload, LoD and
 // per-frame instance state, and the ordering of one frame's kernels.
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -135,6 +136,7 @@ int fail(cs_ctx *c, int code, const char *fmt, ...) {
     do {                                                                                    \
         cudaError_t e_ = (call);                                                            \
         if (e_ != cudaSuccess) {                                                            \
+            cudaGetLastError(); /* reported here, not again by the next call */             \
             return fail(ctx, e_ == cudaErrorMemoryAllocation ? CS_ERR_OOM : CS_ERR_CUDA,    \
                         "%s failed: %s (%s:%d)", #call, cudaGetErrorString(e_), __FILE__,  \
                         __LINE__);                                                          \
@@ -360,15 +362,32 @@ void cam_params(const cs_ctx *c, const cs_camera *cam, CamParams &p) {
     }
 }
 
-// Device memory of the context's GPU (a kernel may read it; other memory goes
-// through cudaMemcpyAsync).
-bool on_this_device(const cs_ctx *ctx, const void *p) {
+// Device memory of the context's GPU whose allocation holds `bytes` bytes from
+// p on: a kernel may read it.  Other memory goes through cudaMemcpyAsync,
+// which also refuses what is not there.
+bool on_this_device(const cs_ctx *ctx, const void *p, size_t bytes) {
+    // (the driver's call; the library links only the runtime)
+    using AddressRange = CUresult (*)(CUdeviceptr *, size_t *, CUdeviceptr);
+    static const AddressRange address_range = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<AddressRange>(f);
+    }();
     cudaPointerAttributes at{};
-    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    if (!address_range || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    return at.type == cudaMemoryTypeDevice && at.device == ctx->device;
+    if (at.type != cudaMemoryTypeDevice || at.device != ctx->device) return false;
+    const CUdeviceptr at_p = reinterpret_cast<CUdeviceptr>(p);
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    return address_range(&base, &size, at_p) == CUDA_SUCCESS && bytes <= size && at_p - base <= size - bytes;
 }
 
 // Add the stage times of event set k (a completed frame) to the running sums.
@@ -850,8 +869,9 @@ int cs_set_instances(cs_ctx *ctx, int32_t n, const int32_t *template_id, const f
         }
         const bool words = ((reinterpret_cast<uintptr_t>(template_id) | reinterpret_cast<uintptr_t>(root) |
                              reinterpret_cast<uintptr_t>(joint_pose)) & 3u) == 0;
-        if (on_device && words && on_this_device(ctx, template_id) && on_this_device(ctx, root) &&
-            on_this_device(ctx, joint_pose)) {
+        if (on_device && words && on_this_device(ctx, template_id, sizeof(int32_t) * n) &&
+            on_this_device(ctx, root, sizeof(float) * 12 * n) &&
+            on_this_device(ctx, joint_pose, sizeof(float) * kJoints * 3 * n)) {
             launch_copy_instances(n, template_id, root, joint_pose, ctx->tid.p, ctx->root.p, ctx->pose.p, ctx->stream);
             CS_CUDA(cudaGetLastError());
         } else {
