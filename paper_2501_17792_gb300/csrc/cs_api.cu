@@ -20,6 +20,7 @@
 #include "../../include/crowdsplat_lod.h"
 #include "../../include/crowdsplat_grad.h"
 #include "cs_internal.cuh"
+#include "cs_poll.cuh"
 
 using namespace cs;
 
@@ -420,9 +421,14 @@ int accumulate_stage_times(cs_ctx *ctx, int k) {
 // 256x256 takes 196 us instead of 218, of 100 x 12,661 Gaussians at 1280x720
 // 461 instead of 496.
 int wait_counts(cs_ctx *ctx, const void *flag, uint32_t seq) {
-    for (int i = 0; i < 1 << 20; ++i)
-        if (__atomic_load_n(static_cast<const uint32_t *>(flag), __ATOMIC_ACQUIRE) == seq) return CS_OK;
-    CS_CUDA(cudaStreamSynchronize(ctx->stream));
+    cudaError_t e = cudaSuccess;
+    const Arrival a = wait_for(static_cast<const uint32_t *>(flag), seq, 1 << 20, [&] {
+        e = cudaStreamSynchronize(ctx->stream);
+        return e == cudaSuccess;
+    });
+    CS_CUDA(e);
+    // counts of an earlier frame would size this one's buffers
+    if (a != Arrival::kThere) return fail(ctx, CS_ERR_CUDA, "the frame's counts were not written");
     return CS_OK;
 }
 
