@@ -16,15 +16,15 @@ int main() {
     auto done = [&] { ++waits; return true; };
     auto writes = [&] { ++waits; flag = 7; return true; };
     auto fails = [&] { ++waits; flag = 7; return false; };
+    auto report = [&](cs::Arrival a) { std::printf("%d %d ", (int)a, waits); };
     // never written, although the stream has finished
-    std::printf("%d", (int)cs::wait_for(&flag, 7u, 100, done));
-    std::printf(" %d", waits);
+    report(cs::wait_for(&flag, 7u, 100, done));
     // written while the stream was waited for
-    std::printf(" %d %d", (int)cs::wait_for(&flag, 7u, 100, writes), waits);
+    report(cs::wait_for(&flag, 7u, 100, writes));
     // there at once: the stream is not waited for
-    std::printf(" %d %d", (int)cs::wait_for(&flag, 7u, 100, done), waits);
+    report(cs::wait_for(&flag, 7u, 100, done));
     flag = 6;
-    std::printf(" %d %d\n", (int)cs::wait_for(&flag, 7u, 0, fails), waits);
+    report(cs::wait_for(&flag, 7u, 0, fails));
 }
 """
 
