@@ -122,15 +122,23 @@ int cs_mlp_forward(cs_mlp *m, int64_t n, const float *feat, const int32_t *band,
  * *loss_out (HOST, may be NULL) receives the batch loss before the step
  * (the call then synchronises the stream).  Errors: CS_ERR_ARG (n < 1,
  * lr <= 0, NULL or misaligned arrays), CS_ERR_OOM, CS_ERR_CUDA (also when
- * the training kernel gave up waiting for its products: the parameters then
- * keep their values until cs_mlp_set_params). */
+ * the training kernel gave up waiting for its products or inputs).  After a
+ * step that gave up the parameters stay those before it; a call without
+ * loss_out does not wait, so the next cs_mlp_train_step, cs_mlp_get_grad or
+ * cs_mlp_get_params reports it (CS_ERR_CUDA; get_params still writes the
+ * parameters), and so do all until cs_mlp_set_params. */
 int cs_mlp_train_step(cs_mlp *m, int64_t n, const float *feat, const int32_t *band, const float *target,
                       float lr, float *loss_out);
 
 /* FP32 gradient of the last cs_mlp_train_step (before the Adam update), in
  * the parameter layout; HOST array of CS_MLP_PARAMS floats.  Errors:
- * CS_ERR_STATE before the first step. */
+ * CS_ERR_STATE before the first step, CS_ERR_CUDA after a step that gave up. */
 int cs_mlp_get_grad(cs_mlp *m, float *host_out);
+
+/* Testing hook: while on, a training step's first product is never reported
+ * as complete, so the step gives up after its bounded waits (about two
+ * seconds). */
+int cs_debug_mlp_lose_product(cs_mlp *m, int32_t on);
 
 #ifdef __cplusplus
 }

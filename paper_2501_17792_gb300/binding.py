@@ -108,6 +108,7 @@ SIGNATURES = {
     "cs_mlp_forward": (C.c_int, [_P, C.c_int64, _P, _P, _P]),
     "cs_mlp_train_step": (C.c_int, [_P, C.c_int64, _P, _P, _P, C.c_float, C.POINTER(C.c_float)]),
     "cs_mlp_get_grad": (C.c_int, [_P, _P]),
+    "cs_debug_mlp_lose_product": (C.c_int, [_P, C.c_int32]),
     # gradients (include/crowdsplat_grad.h)
     "cs_render_train": (C.c_int, [_P, C.POINTER(Camera), _P, C.POINTER(FrameStats)]),
     "cs_backward": (C.c_int, [_P, _P, C.POINTER(Grads)]),

@@ -271,11 +271,14 @@ constexpr uint32_t kTcOffW = kTcGroups * kTcGroupBytes;
 constexpr uint32_t kTcOffStage = kTcOffW + 3 * kTcWBuf;
 static_assert(kTcStage % 128 == 0, "alignment of what follows");
 constexpr uint32_t kTcOffVec = kTcOffStage + kTcGroups * kTcStage;  // b1, b2, w3, b3
-constexpr uint32_t kTcOffBar = kTcOffVec + (3 * kH + 4) * 4;        // mbarriers, TMEM address, fail flags
+constexpr uint32_t kTcOffBar = kTcOffVec + (3 * kH + 4) * 4;        // mbarriers, TMEM address
 constexpr size_t kSmemTc = kTcOffBar + 64 + 1024;                   // (1,024: alignment)
 static_assert(kSmemTc <= 227 * 1024, "shared memory of the training kernel");
 constexpr uint32_t kTcCols = 512;  // TMEM columns: 64 per group for Z, 128 per group for G (from 128 on)
-constexpr long long kTcWaitClocks = 4000000000ll;  // a wait gives up after about two seconds
+// a wait gives up after about a second, and not before it has polled some more
+// (the clock also runs while the context is switched out)
+constexpr long long kTcWaitClocks = 2000000000ll;
+constexpr int kTcLatePolls = 256;
 
 // matrix descriptor (128-byte swizzle): start address, stride between the
 // 64-column halves of an MN-major operand, 1,024 bytes between 8-row groups
@@ -304,11 +307,22 @@ __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence:
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void group_sync(int group) { asm volatile("bar.sync %0, 256;" ::"r"(group + 1) : "memory"); }
+// The same barrier; whether a thread of the group came with `failed` (the same
+// answer in all of them).
+__device__ __forceinline__ bool group_failed(int group, uint32_t failed) {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %2, 0;\n\tbar.red.or.pred q, %1, 256, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(r)
+        : "r"(group + 1), "r"(failed)
+        : "memory");
+    return r != 0u;
+}
 
 // Waits for phase `parity` of the mbarrier; false after kTcWaitClocks.
 __device__ __forceinline__ bool tc_wait(uint32_t bar, uint32_t parity) {
     const long long t0 = clock64();
-    for (;;) {
+    for (int late = 0;;) {
         uint32_t done;
         asm volatile(
             "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
@@ -316,7 +330,7 @@ __device__ __forceinline__ bool tc_wait(uint32_t bar, uint32_t parity) {
             : "r"(bar), "r"(parity)
             : "memory");
         if (done) return true;
-        if (clock64() - t0 > kTcWaitClocks) return false;
+        if (clock64() - t0 > kTcWaitClocks && ++late > kTcLatePolls) return false;
     }
 }
 
@@ -408,8 +422,8 @@ __device__ __forceinline__ void tc_input(unsigned char *x, const unsigned char *
 
 __global__ void __launch_bounds__(kTcThreads, 1)
     k_mlp_train(int64_t n, int n_tiles, const float *__restrict__ feat, const int32_t *__restrict__ band,
-                const float *__restrict__ target, Weights W, float inv_n, bool bulk, float *__restrict__ partial,
-                uint32_t *__restrict__ err) {
+                const float *__restrict__ target, Weights W, float inv_n, bool bulk, bool lose, float *__restrict__ partial,
+                uint32_t *__restrict__ err, volatile uint32_t *host_err) {
     extern __shared__ unsigned char tc_raw[];
     unsigned char *smem = tc_raw + ((1024u - ((uint32_t)__cvta_generic_to_shared(tc_raw) & 1023u)) & 1023u);
     // t: thread of the group; r: its row of the tile, half: its half of the hidden units
@@ -423,7 +437,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                      *vw3 = reinterpret_cast<const ulonglong2 *>(sw3);  // four values each
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kTcOffBar);
     uint32_t *s_tmem = reinterpret_cast<uint32_t *>(bars + 2 * kTcGroups);
-    volatile uint32_t *s_fail = s_tmem + 1;  // per group
     // of a group: its products, its staged features
     const uint32_t bar = (uint32_t)__cvta_generic_to_shared(bars + group), stage_bar = bar + 8 * kTcGroups;
 
@@ -448,7 +461,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         sb3[0] = W.master[oB3];
         for (int g = 0; g < 2 * kTcGroups; ++g)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((uint32_t)__cvta_generic_to_shared(bars + g)) : "memory");
-        for (int g = 0; g < kTcGroups; ++g) s_fail[g] = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
@@ -477,55 +489,69 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 #pragma unroll
     for (int i = 0; i < kMine / 2; ++i) s_w3[i] = s_b2[i] = s_b1[i] = 0ull;
     float acc_loss = 0.f, acc_b3 = 0.f;
-    uint32_t phase = 0;
     bool any = false;  // a tile has been added to G
     const int first = (int)blockIdx.x * kTcGroups + group, step = (int)gridDim.x * kTcGroups;
 
     // the first tile's inputs and first product
     int nband = -1;
     float ntarget = 0.f;
-    uint32_t stage_phase = 0;
     auto next_row = [&](int64_t row) {  // band and target of the thread's row of a coming tile
         nband = row < n ? __ldg(band + row) : -1;
         ntarget = row < n ? __ldg(target + row) : 0.f;
     };
+    // A wait that gives up leaves its phase as it is and is noted in the flags;
+    // the group's next barrier tells all its threads, which then leave.
+    // One register of flags: the phases to wait for, a copy that may be in
+    // flight, what was given up, and that the group has left.
+    constexpr uint32_t kPhase = 1u, kStagePhase = 2u, kStaging = 4u, kLostProduct = 8u, kLostStage = 16u, kLeft = 32u;
+    constexpr uint32_t kLost = kLostProduct | kLostStage;
+    uint32_t flags = 0;
     auto staged = [&] {  // the staged features are there
         if (!bulk) {
             group_sync(group);
+            flags &= ~kStaging;
+        } else if (tc_wait(stage_bar, (flags / kStagePhase) & 1u)) {
+            flags = (flags ^ kStagePhase) & ~kStaging;
         } else {
-            if (!tc_wait(stage_bar, stage_phase)) s_fail[group] = 1u;
-            stage_phase ^= 1u;
+            flags |= kLostStage;
         }
+        __syncwarp();
+    };
+    auto product = [&] {  // the last committed product is there
+        flags = tc_wait(bar, flags & kPhase) ? flags ^ kPhase : flags | kLostProduct;
+        __syncwarp();
+        tc_fence_after();
     };
     if (first < n_tiles) {
         const int64_t row0 = (int64_t)first * kTcRows;
+        flags |= kStaging;
         tc_stage(stage, stage_bar, bulk, row0, n, t, feat);
         next_row(row0 + r);
         staged();
         tc_input(sX, stage, row0, n, t, nband);
         tc_fence_smem();
         tc_fence_before();
-        group_sync(group);
-        if (first + step < n_tiles) tc_stage(stage, stage_bar, bulk, (int64_t)(first + step) * kTcRows, n, t, feat);
-        if (issuer) {
+        if (group_failed(group, flags & kLost)) {
+            flags |= kLeft;
+        } else if (first + step < n_tiles) {
+            flags |= kStaging;
+            tc_stage(stage, stage_bar, bulk, (int64_t)(first + step) * kTcRows, n, t, feat);
+        }
+        if (issuer && !(flags & kLeft)) {
             tc_fence_after();
 #pragma unroll
             for (int k = 0; k < kIn / 16; ++k) tc_mma(z_cols, tc_desc(aX + 32 * k, 0), tc_desc(aW + 32 * k, 0), kFwd, k > 0);
-            tc_commit(bar);
+            if (!(lose && tid == 0 && blockIdx.x == 0)) tc_commit(bar);
         }
     }
     int xbuf = 0;
-    bool staging = first + step < n_tiles;  // a copy may be in flight
-    for (int tile = first; tile < n_tiles; tile += step, xbuf ^= 1) {
+    for (int tile = first; tile < n_tiles && !(flags & kLeft); tile += step, xbuf ^= 1) {
         const bool valid = (int64_t)tile * kTcRows + r < n, more = tile + step < n_tiles;
         const int64_t next0 = (int64_t)(tile + step) * kTcRows;
         const float y_target = ntarget;
         if (more) next_row(next0 + r);
         // ---- h1 = relu(Z1 + b1) ------------------------------------------
-        if (!tc_wait(bar, phase)) s_fail[group] = 1u;
-        phase ^= 1u;
-        __syncwarp();
-        tc_fence_after();
+        product();
 #pragma unroll
         for (int c0 = 0; c0 < kMine; c0 += 16) {
             f2 z[8];
@@ -542,8 +568,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         }
         tc_fence_smem();
         tc_fence_before();
-        group_sync(group);
-        if (s_fail[group]) break;  // the same for the whole group: set before the barrier
+        if (group_failed(group, flags & kLost)) {
+            flags |= kLeft;
+            break;
+        }
         if (issuer) {
             tc_fence_after();
 #pragma unroll
@@ -554,14 +582,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         // the next tile's inputs, while Z2 is computed
         if (more) {
             staged();
-            staging = false;
             tc_input(sX + (xbuf ^ 1) * kTcBuf, stage, next0, n, t, nband);
         }
         // ---- y, dy, dz2 = dy w3 [z2 > 0] ---------------------------------
-        if (!tc_wait(bar, phase)) s_fail[group] = 1u;
-        phase ^= 1u;
-        __syncwarp();
-        tc_fence_after();
+        product();
         f2 y2 = 0ull;
 #pragma unroll
         for (int c0 = 0; c0 < kMine; c0 += 16) {
@@ -604,10 +628,14 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         }
         tc_fence_smem();
         tc_fence_before();
-        group_sync(group);
-        if (s_fail[group]) break;
-        staging = tile + 2 * step < n_tiles;
-        if (staging) tc_stage(stage, stage_bar, bulk, (int64_t)(tile + 2 * step) * kTcRows, n, t, feat);
+        if (group_failed(group, flags & kLost)) {
+            flags |= kLeft;
+            break;
+        }
+        if (tile + 2 * step < n_tiles) {
+            flags |= kStaging;
+            tc_stage(stage, stage_bar, bulk, (int64_t)(tile + 2 * step) * kTcRows, n, t, feat);
+        }
         if (issuer) {
             tc_fence_after();
 #pragma unroll
@@ -616,10 +644,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             tc_commit(bar);
         }
         // ---- dz1 = dH1 [h1 > 0] ------------------------------------------
-        if (!tc_wait(bar, phase)) s_fail[group] = 1u;
-        phase ^= 1u;
-        __syncwarp();
-        tc_fence_after();
+        product();
 #pragma unroll
         for (int c0 = 0; c0 < kMine; c0 += 16) {
             f2 z[8];
@@ -638,8 +663,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         }
         tc_fence_smem();
         tc_fence_before();
-        group_sync(group);
-        if (s_fail[group]) break;
+        if (group_failed(group, flags & kLost)) {
+            flags |= kLeft;
+            break;
+        }
         if (issuer) {
             tc_fence_after();
             // G, sixteen rows a product: [H1 | X] and [dZ2 | dZ1]
@@ -656,11 +683,24 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         }
         any = true;
     }
-    if (bulk && staging) tc_wait(stage_bar, stage_phase);  // (after a failed wait only)
-    if (any && !s_fail[group] && !tc_wait(bar, phase)) s_fail[group] = 1u;
-    __syncwarp();
+    if (any && !(flags & kLeft)) product();
+    // after a wait that gave up: what is still in flight reads or writes
+    // shared memory and TMEM (a second wait, with the same limit)
+    if (flags & kLostProduct) tc_wait(bar, flags & kPhase);
+    if (bulk && (flags & kStaging)) tc_wait(stage_bar, (flags / kStagePhase) & 1u);
+    tc_fence_before();
+    const bool bad = __syncthreads_or((int)(flags & kLost));
     tc_fence_after();
-    __syncthreads();
+    if (bad) {
+        // no gradient: the host is told, the parameters stay
+        if (tid == 0) {
+            atomicOr(err, 1u);
+            *host_err = 1u;
+        }
+        __syncwarp();
+        if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcCols) : "memory");
+        return;
+    }
 
     // ---- per-CTA partial gradient, written in a fixed order --------------
     // the groups' G: a row's two threads read half of its columns each; group
@@ -731,7 +771,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                                                                           : tid == 3 * kH ? oB3 : kP;
         out[o] = a;  // (kP: the sum of squared errors)
     }
-    if (t == 0 && s_fail[group]) atomicOr(err, 1u);
     tc_fence_before();
     __syncthreads();
     if (warp == 0) {
@@ -822,6 +861,9 @@ struct cs_mlp {
     float *partial = nullptr;
     int n_part_cap = 0;
     int64_t steps = 0;
+    bool lose_product = false;  // cs_debug_mlp_lose_product
+    // set by a training kernel that gave up waiting (pinned)
+    volatile uint32_t *gave_up() const { return reinterpret_cast<volatile uint32_t *>(h_sse + 2); }
 };
 
 namespace {
@@ -834,6 +876,11 @@ int mfail(cs_mlp *m, int code, const char *fmt, ...) {
     va_end(ap);
     m->err = buf;
     return code;
+}
+
+int failed_step(cs_mlp *m) {
+    return mfail(m, CS_ERR_CUDA, "a training step gave up waiting for its tensor-core products or inputs: the parameters "
+                 "are those before it (cs_mlp_set_params to go on)");
 }
 
 #define MLP_CUDA(m, call)                                                                         \
@@ -928,7 +975,7 @@ int cs_mlp_get_params(cs_mlp *m, float *host_out) {
     MLP_CUDA(m, cudaSetDevice(m->device));
     MLP_CUDA(m, cudaMemcpyAsync(host_out, m->master, kP * 4, cudaMemcpyDeviceToHost, m->stream));
     MLP_CUDA(m, cudaStreamSynchronize(m->stream));
-    return CS_OK;
+    return *m->gave_up() ? failed_step(m) : CS_OK;
 }
 
 int cs_mlp_set_params(cs_mlp *m, const float *host_in) {
@@ -944,6 +991,7 @@ int cs_mlp_set_params(cs_mlp *m, const float *host_in) {
     int rc = refresh_copies(m);
     if (rc != CS_OK) return rc;
     MLP_CUDA(m, cudaStreamSynchronize(m->stream));
+    *m->gave_up() = 0u;
     m->steps = 0;
     return CS_OK;
 }
@@ -971,6 +1019,7 @@ int cs_mlp_train_step(cs_mlp *m, int64_t n, const float *feat, const int32_t *ba
     if (!(lr > 0.0f) || !std::isfinite(lr)) return mfail(m, CS_ERR_ARG, "lr must be > 0");
     if (!feat || !band || !target || !aligned(feat, 8) || !aligned(band, 4) || !aligned(target, 4))
         return mfail(m, CS_ERR_ARG, "NULL or misaligned array");
+    if (*m->gave_up()) return failed_step(m);
     MLP_CUDA(m, cudaSetDevice(m->device));
     const int grid = grid_for(m, n, kTcGroups * kTcRows, 1);
     if (grid > m->n_part_cap) {
@@ -985,7 +1034,8 @@ int cs_mlp_train_step(cs_mlp *m, int64_t n, const float *feat, const int32_t *ba
     Weights W{m->w1t, m->w2t, m->w2n, m->master};
     uint32_t *err = reinterpret_cast<uint32_t *>(m->sse + 1);
     k_mlp_train<<<grid, kTcThreads, kSmemTc, m->stream>>>(n, tiles, feat, band, target, W, (float)(1.0 / (double)n),
-                                                          aligned(feat, 16), m->partial, err);
+                                                          aligned(feat, 16), m->lose_product, m->partial, err,
+                                                          m->gave_up());
     MLP_CUDA(m, cudaGetLastError());
     const int64_t t = m->steps + 1;
     const float bc1 = (float)(1.0 - std::pow(0.9, (double)t)), bc2 = (float)(1.0 - std::pow(0.999, (double)t));
@@ -994,11 +1044,12 @@ int cs_mlp_train_step(cs_mlp *m, int64_t n, const float *feat, const int32_t *ba
     MLP_CUDA(m, cudaGetLastError());
     m->steps = t;
     if (loss_out) {
-        MLP_CUDA(m, cudaMemcpyAsync(m->h_sse, m->sse, 8, cudaMemcpyDeviceToHost, m->stream));
+        MLP_CUDA(m, cudaMemcpyAsync(m->h_sse, m->sse, 4, cudaMemcpyDeviceToHost, m->stream));
         MLP_CUDA(m, cudaStreamSynchronize(m->stream));
-        uint32_t failed;
-        std::memcpy(&failed, m->h_sse + 1, 4);
-        if (failed) return mfail(m, CS_ERR_CUDA, "the training kernel gave up waiting for its tensor-core products");
+        if (*m->gave_up()) {
+            m->steps = t - 1;
+            return failed_step(m);
+        }
         *loss_out = (float)((double)m->h_sse[0] / (double)n);
     }
     return CS_OK;
@@ -1007,10 +1058,16 @@ int cs_mlp_train_step(cs_mlp *m, int64_t n, const float *feat, const int32_t *ba
 int cs_mlp_get_grad(cs_mlp *m, float *host_out) {
     if (!m) return CS_ERR_ARG;
     if (!host_out) return mfail(m, CS_ERR_ARG, "NULL output");
-    if (m->steps == 0) return mfail(m, CS_ERR_STATE, "no training step yet");
+    if (m->steps == 0 && !*m->gave_up()) return mfail(m, CS_ERR_STATE, "no training step yet");
     MLP_CUDA(m, cudaSetDevice(m->device));
     MLP_CUDA(m, cudaMemcpyAsync(host_out, m->grad, kP * 4, cudaMemcpyDeviceToHost, m->stream));
     MLP_CUDA(m, cudaStreamSynchronize(m->stream));
+    return *m->gave_up() ? failed_step(m) : CS_OK;
+}
+
+int cs_debug_mlp_lose_product(cs_mlp *m, int32_t on) {
+    if (!m) return CS_ERR_ARG;
+    m->lose_product = on != 0;
     return CS_OK;
 }
 
