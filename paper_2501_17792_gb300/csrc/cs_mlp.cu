@@ -254,12 +254,22 @@ __global__ void __launch_bounds__(kThreads, 2)
 //
 // Bound by latency (issue slots 45%, shared-memory and TMEM data path 47%,
 // tensor pipe 17%): a group's three waits per tile and its loads from TMEM,
-// with two groups an SM, which shared memory (100 KB each) and TMEM (192
-// columns each) allow.  A training step of 2,752,512 rows: 541 us with
-// mma.sync (weights, activations and gradients as fragments from shared
-// memory, 503 us of it this kernel) -> 412 us (372).  One thread per row
-// instead of two 429; the features by 8-byte cp.async 432; FP32 operations
-// one by one and BF16 conversions one by one 466.
+// with two groups an SM: a thread's 128 registers (96 of them column sums)
+// leave no room for a third, nor do 100 KB of shared memory and 192 TMEM
+// columns each.  A training step of 2,752,512 rows: 541 us with mma.sync
+// (weights, activations and gradients as fragments from shared memory, 503 us
+// of it this kernel) -> 412 us (372).  One thread per row instead of two 429;
+// the features by 8-byte cp.async 432; FP32 operations one by one and BF16
+// conversions one by one 466.
+//
+// Steps of a few thousand rows pay for what a CTA does once: one tile per CTA
+// while there are SMs for that, the first features under way before the
+// weights are read, column sums in 31 shuffles a warp instead of 160 per 32
+// columns, the gradient through shared memory to consecutive addresses, the
+// loss written to the host's memory by the update.  A step and its loss at
+// 3,000 rows 52 -> 36 us, 19,456 rows 52 -> 37, without the loss 39 -> 29 and
+// 41 -> 30; 300,000 rows 76.9 -> 65.1, 2,752,512 rows 390 -> 372.  (128-row
+// tiles with mma.sync, one tile per SM: 41, 44; 30, 34; 104, 690.)
 // ---------------------------------------------------------------------------
 
 constexpr int kTcGroups = 2, kTcGroupThreads = 256, kTcThreads = kTcGroupThreads * kTcGroups, kTcRows = 128;
@@ -420,6 +430,28 @@ __device__ __forceinline__ void tc_input(unsigned char *x, const unsigned char *
     }
 }
 
+// Lane l's result: the sum over the warp's lanes of value l of their 32 (half of
+// what is left is sent and received at each step: 31 shuffles in place of 160).
+__device__ __forceinline__ float lane_column_sum(const f2 (&v)[16]) {
+    const int lane = threadIdx.x & 31;
+    float x[32];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        x[2 * i] = lo2(v[i]);
+        x[2 * i + 1] = hi2(v[i]);
+    }
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) {
+        const bool upper = (lane & s) != 0;
+#pragma unroll
+        for (int i = 0; i < s; ++i) {
+            const float got = __shfl_xor_sync(0xffffffffu, upper ? x[i] : x[i + s], s);
+            x[i] = (upper ? x[i + s] : x[i]) + got;
+        }
+    }
+    return x[0];
+}
+
 __global__ void __launch_bounds__(kTcThreads, 1)
     k_mlp_train(int64_t n, int n_tiles, const float *__restrict__ feat, const int32_t *__restrict__ band,
                 const float *__restrict__ target, Weights W, float inv_n, bool bulk, bool lose, float *__restrict__ partial,
@@ -440,29 +472,41 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     // of a group: its products, its staged features
     const uint32_t bar = (uint32_t)__cvta_generic_to_shared(bars + group), stage_bar = bar + 8 * kTcGroups;
 
-    // weights into the swizzled layout (columns past a row's length zero)
-    for (int i = tid; i < 3 * kH * 8; i += kTcThreads) {
-        const int m = i / (kH * 8), wr = (i >> 3) & (kH - 1), c = i & 7;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (m == 0) {
-            if (c < kIn / 8) v = *reinterpret_cast<const uint4 *>(W.w1t + wr * kLdW1 + 8 * c);
-        } else {
-            v = *reinterpret_cast<const uint4 *>((m == 1 ? W.w2t : W.w2n) + wr * kLdW2 + 8 * c);
-        }
-        *tc_chunk(sW + m * kTcWBuf, wr, c) = v;
+    // the group's first features start before the weights are read
+    const int first = (int)blockIdx.x + group * (int)gridDim.x, step = (int)gridDim.x * kTcGroups;
+    const int64_t first0 = (int64_t)first * kTcRows;
+    if (t == 32) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(stage_bar) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        tc_fence_smem();
     }
-    for (int i = tid; i < kH; i += kTcThreads) {
-        sb1[i] = W.master[oB1 + i];
-        sb2[i] = W.master[oB2 + i];
-        sw3[i] = W.master[oW3 + i];
+    int nband = -1;
+    float ntarget = 0.f;
+    auto next_row = [&](int64_t row) {  // band and target of the thread's row of a coming tile
+        nband = row < n ? __ldg(band + row) : -1;
+        ntarget = row < n ? __ldg(target + row) : 0.f;
+    };
+    if (first < n_tiles) {
+        tc_stage(stage, stage_bar, bulk, first0, n, t, feat);
+        next_row(first0 + r);
+    }
+    // weights into the swizzled layout (columns past a row's length zero), one
+    // 16-byte chunk of each matrix a thread
+    {
+        static_assert(kTcThreads == kH * 8, "a chunk per thread");
+        const int wr = tid >> 3, c = tid & 7;
+        uint4 v1 = make_uint4(0u, 0u, 0u, 0u);
+        if (c < kIn / 8) v1 = *reinterpret_cast<const uint4 *>(W.w1t + wr * kLdW1 + 8 * c);
+        const uint4 v2 = *reinterpret_cast<const uint4 *>(W.w2t + wr * kLdW2 + 8 * c);
+        const uint4 v3 = *reinterpret_cast<const uint4 *>(W.w2n + wr * kLdW2 + 8 * c);
+        if (tid < 3 * kH) sb1[tid] = W.master[(tid < kH ? oB1 : tid < 2 * kH ? oB2 - kH : oW3 - 2 * kH) + tid];
+        if (tid == 3 * kH) sb3[0] = W.master[oB3];
+        *tc_chunk(sW, wr, c) = v1;
+        *tc_chunk(sW + kTcWBuf, wr, c) = v2;
+        *tc_chunk(sW + 2 * kTcWBuf, wr, c) = v3;
     }
     for (int c = 5; c < 8; ++c) *tc_chunk(sX + half * kTcBuf, r, c) = make_uint4(0u, 0u, 0u, 0u);
-    if (tid == 0) {
-        sb3[0] = W.master[oB3];
-        for (int g = 0; g < 2 * kTcGroups; ++g)
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((uint32_t)__cvta_generic_to_shared(bars + g)) : "memory");
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
     if (warp == 0) {
         __syncwarp();
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -490,22 +534,15 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     for (int i = 0; i < kMine / 2; ++i) s_w3[i] = s_b2[i] = s_b1[i] = 0ull;
     float acc_loss = 0.f, acc_b3 = 0.f;
     bool any = false;  // a tile has been added to G
-    const int first = (int)blockIdx.x * kTcGroups + group, step = (int)gridDim.x * kTcGroups;
 
     // the first tile's inputs and first product
-    int nband = -1;
-    float ntarget = 0.f;
-    auto next_row = [&](int64_t row) {  // band and target of the thread's row of a coming tile
-        nband = row < n ? __ldg(band + row) : -1;
-        ntarget = row < n ? __ldg(target + row) : 0.f;
-    };
     // A wait that gives up leaves its phase as it is and is noted in the flags;
     // the group's next barrier tells all its threads, which then leave.
     // One register of flags: the phases to wait for, a copy that may be in
     // flight, what was given up, and that the group has left.
     constexpr uint32_t kPhase = 1u, kStagePhase = 2u, kStaging = 4u, kLostProduct = 8u, kLostStage = 16u, kLeft = 32u;
     constexpr uint32_t kLost = kLostProduct | kLostStage;
-    uint32_t flags = 0;
+    uint32_t flags = first < n_tiles ? kStaging : 0u;
     auto staged = [&] {  // the staged features are there
         if (!bulk) {
             group_sync(group);
@@ -523,12 +560,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         tc_fence_after();
     };
     if (first < n_tiles) {
-        const int64_t row0 = (int64_t)first * kTcRows;
-        flags |= kStaging;
-        tc_stage(stage, stage_bar, bulk, row0, n, t, feat);
-        next_row(row0 + r);
         staged();
-        tc_input(sX, stage, row0, n, t, nband);
+        tc_input(sX, stage, first0, n, t, nband);
         tc_fence_smem();
         tc_fence_before();
         if (group_failed(group, flags & kLost)) {
@@ -703,70 +736,54 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     }
 
     // ---- per-CTA partial gradient, written in a fixed order --------------
-    // the groups' G: a row's two threads read half of its columns each; group
-    // 1 leaves its quarters in shared memory (over the activations), group 0
-    // adds them
+    // Over the activations: each group's quarters of G (a row's two threads
+    // read half of its columns each) and its warps' column sums; then
+    // consecutive threads write consecutive values.  A group without a tile
+    // has neither.
     float *out = partial + (size_t)blockIdx.x * (kP + 1);
-    constexpr int kLdG = 65;
-    float *sG = reinterpret_cast<float *>(smem);            // [128][kLdG]
-    float *sRed = sG + 128 * kLdG;                          // [8 warp rows][3 kH + 2]
+    constexpr int kLdG = kH + 1, kGFloats = 2 * kH * kLdG;
+    float *sG = reinterpret_cast<float *>(smem);            // [groups][128][kLdG]
+    float *sRed = sG + kTcGroups * kGFloats;                // [8 warp rows][3 kH + 2]
     constexpr int kLdR = 3 * kH + 2;
-    const uint32_t my_g = g_cols + my_lanes + (r < kH ? 0 : kH) + mine;  // dW2's columns, dW1's
-#pragma unroll
-    for (int c0 = 0; c0 < kMine; c0 += 16) {
-        f2 z[8];
+    const bool both = (int)(blockIdx.x + gridDim.x) < n_tiles;  // the second group had a tile
+    if (any) {
         // (warps 0, 1, 4 and 5 of a group hold dW2's rows, the others dW1's)
-        tc_load16(z, my_g + c0);
-        if (group == 1) {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) sG[r * kLdG + mine + c0 + i] = any ? (i & 1 ? hi2(z[i / 2]) : lo2(z[i / 2])) : 0.f;
-        }
-    }
-    float *red = sRed + (4 * group + (warp & 3)) * kLdR;  // 32 rows of the tiles, both halves' columns
-#pragma unroll
-    for (int i = 0; i < kMine; ++i) {
-        float a = i & 1 ? hi2(s_w3[i / 2]) : lo2(s_w3[i / 2]), b = i & 1 ? hi2(s_b2[i / 2]) : lo2(s_b2[i / 2]),
-              c = i & 1 ? hi2(s_b1[i / 2]) : lo2(s_b1[i / 2]);
-#pragma unroll
-        for (int s = 1; s < 32; s <<= 1) {
-            a += __shfl_xor_sync(0xffffffffu, a, s);
-            b += __shfl_xor_sync(0xffffffffu, b, s);
-            c += __shfl_xor_sync(0xffffffffu, c, s);
-        }
-        if (lane == 0) {
-            red[mine + i] = a;
-            red[kH + mine + i] = b;
-            red[2 * kH + mine + i] = c;
-        }
-    }
-    float l = acc_loss, b3 = acc_b3;
-#pragma unroll
-    for (int s = 1; s < 32; s <<= 1) {
-        l += __shfl_xor_sync(0xffffffffu, l, s);
-        b3 += __shfl_xor_sync(0xffffffffu, b3, s);
-    }
-    if (lane == 0 && half == 0) {
-        red[3 * kH] = b3;
-        red[3 * kH + 1] = l;
-    }
-    __syncthreads();
-    if (group == 0) {
+        const uint32_t my_g = g_cols + my_lanes + (r < kH ? 0 : kH) + mine;  // dW2's columns, dW1's
+        float *row = sG + group * kGFloats + r * kLdG + mine;
 #pragma unroll
         for (int c0 = 0; c0 < kMine; c0 += 16) {
             f2 z[8];
             tc_load16(z, my_g + c0);
-            // row r of dW2, row r - 64 of dW1 (its rows past kIn are padding)
-            if (r < kH + kIn) {
-                float *o = out + (r < kH ? oW2 + r * kH : oW1 + (r - kH) * kH) + mine + c0;
 #pragma unroll
-                for (int i = 0; i < 16; ++i)
-                    o[i] = (any ? (i & 1 ? hi2(z[i / 2]) : lo2(z[i / 2])) : 0.f) + sG[r * kLdG + mine + c0 + i];
+            for (int i = 0; i < 8; ++i) {
+                row[c0 + 2 * i] = lo2(z[i]);
+                row[c0 + 2 * i + 1] = hi2(z[i]);
             }
         }
+        float *red = sRed + (4 * group + (warp & 3)) * kLdR;  // 32 rows of the tiles, both halves' columns
+        red[mine + lane] = lane_column_sum(s_w3);
+        red[kH + mine + lane] = lane_column_sum(s_b2);
+        red[2 * kH + mine + lane] = lane_column_sum(s_b1);
+        float l = acc_loss, b3 = acc_b3;
+#pragma unroll
+        for (int s = 1; s < 32; s <<= 1) {
+            l += __shfl_xor_sync(0xffffffffu, l, s);
+            b3 += __shfl_xor_sync(0xffffffffu, b3, s);
+        }
+        if (lane == 0 && half == 0) {
+            red[3 * kH] = b3;
+            red[3 * kH + 1] = l;
+        }
+    }
+    __syncthreads();
+    // row r of dW2, row r - 64 of dW1 (its rows past kIn are padding)
+    for (int i = tid; i < (kH + kIn) * kH; i += kTcThreads) {
+        const float *g = sG + (i / kH) * kLdG + i % kH;
+        out[i < kH * kH ? oW2 + i : oW1 + i - kH * kH] = both ? g[0] + g[kGFloats] : g[0];
     }
     if (tid < kLdR) {
         float a = 0.f;
-        for (int w = 0; w < 4 * kTcGroups; ++w) a += sRed[w * kLdR + tid];
+        for (int w = 0; w < (both ? 8 : 4); ++w) a += sRed[w * kLdR + tid];
         const int o = tid < kH ? oW3 + tid : tid < 2 * kH ? oB2 + tid - kH : tid < 3 * kH ? oB1 + tid - 2 * kH
                                                                           : tid == 3 * kH ? oB3 : kP;
         out[o] = a;  // (kP: the sum of squared errors)
@@ -782,7 +799,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 // Sum the per-CTA partials, then Adam on the FP32 master weights and refresh
 // the BF16 copies.  A block takes 32 parameters, a warp a run of the
 // partials; the eight warps' sums are added in order.  Parameter kP is the
-// sum of the squared errors.  After a training kernel that gave up waiting
+// sum of the squared errors, which goes to the host's memory (pinned).  After a training kernel that gave up waiting
 // (*err) the parameters stay as they are.  One thread per parameter over all
 // 152 partials took 16 us (a chain of loads).
 constexpr int kAdamWarps = 8;
@@ -795,6 +812,10 @@ __global__ void __launch_bounds__(32 * kAdamWarps)
     __shared__ float sums[kAdamWarps][32];
     const int warp = threadIdx.x >> 5, p = blockIdx.x * 32 + (threadIdx.x & 31);
     const int run = (n_part + kAdamWarps - 1) / kAdamWarps, c1 = min(n_part, (warp + 1) * run);
+    // (what the update reads is loaded with the partials, not after them)
+    const bool mine = warp == 0 && p < kP;
+    const float m0 = mine ? m1[p] : 0.f, v0 = mine ? m2[p] : 0.f, th0 = mine ? master[p] : 0.f;
+    const bool failed = *err != 0u;
     float s = 0.f;
     if (p <= kP) {
 #pragma unroll 8
@@ -802,7 +823,7 @@ __global__ void __launch_bounds__(32 * kAdamWarps)
     }
     sums[warp][threadIdx.x & 31] = s;
     __syncthreads();
-    if (warp > 0 || p > kP || *err) return;
+    if (warp > 0 || p > kP || failed) return;
     s = 0.f;
     for (int w = 0; w < kAdamWarps; ++w) s += sums[w][threadIdx.x];
     if (p == kP) {
@@ -811,11 +832,11 @@ __global__ void __launch_bounds__(32 * kAdamWarps)
     }
     grad[p] = s;
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-    const float m = b1 * m1[p] + (1.f - b1) * s;
-    const float v = b2 * m2[p] + (1.f - b2) * s * s;
+    const float m = b1 * m0 + (1.f - b1) * s;
+    const float v = b2 * v0 + (1.f - b2) * s * s;
     m1[p] = m;
     m2[p] = v;
-    const float th = master[p] - lr * (m / bc1) / (sqrtf(v / bc2) + eps);
+    const float th = th0 - lr * (m / bc1) / (sqrtf(v / bc2) + eps);
     master[p] = th;
     if (p < oB1) {
         const int k = p / kH, n = p % kH;
@@ -856,13 +877,14 @@ struct cs_mlp {
     cudaStream_t stream = nullptr;
     int n_sm = 0;
     std::string err;
-    float *master = nullptr, *m1 = nullptr, *m2 = nullptr, *grad = nullptr, *sse = nullptr, *h_sse = nullptr;
+    float *master = nullptr, *m1 = nullptr, *m2 = nullptr, *grad = nullptr, *h_sse = nullptr;
+    uint32_t *failed = nullptr;  // set by a training kernel that gave up waiting: no update
     __nv_bfloat16 *w1t = nullptr, *w2t = nullptr, *w2n = nullptr;
     float *partial = nullptr;
     int n_part_cap = 0;
     int64_t steps = 0;
     bool lose_product = false;  // cs_debug_mlp_lose_product
-    // set by a training kernel that gave up waiting (pinned)
+    // the same for the host (pinned, behind the sum of the squared errors)
     volatile uint32_t *gave_up() const { return reinterpret_cast<volatile uint32_t *>(h_sse + 2); }
 };
 
@@ -926,7 +948,7 @@ int cs_mlp_create(cs_mlp **out, int32_t device, void *stream, uint64_t seed) {
     if (cudaDeviceGetAttribute(&m->n_sm, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return bail(CS_ERR_CUDA);
     if (cudaMalloc(&m->master, kP * 4) != cudaSuccess || cudaMalloc(&m->m1, kP * 4) != cudaSuccess ||
         cudaMalloc(&m->m2, kP * 4) != cudaSuccess || cudaMalloc(&m->grad, kP * 4) != cudaSuccess ||
-        cudaMalloc(&m->sse, 16) != cudaSuccess || cudaMalloc(&m->w1t, kW1Elems * 2) != cudaSuccess ||
+        cudaMalloc(&m->failed, sizeof(uint32_t)) != cudaSuccess || cudaMalloc(&m->w1t, kW1Elems * 2) != cudaSuccess ||
         cudaMalloc(&m->w2t, kW2Elems * 2) != cudaSuccess || cudaMalloc(&m->w2n, kW2Elems * 2) != cudaSuccess ||
         cudaMallocHost(&m->h_sse, 16) != cudaSuccess) {
         cudaGetLastError();
@@ -958,7 +980,7 @@ void cs_mlp_destroy(cs_mlp *m) {
     cudaFree(m->m1);
     cudaFree(m->m2);
     cudaFree(m->grad);
-    cudaFree(m->sse);
+    cudaFree(m->failed);
     cudaFree(m->w1t);
     cudaFree(m->w2t);
     cudaFree(m->w2n);
@@ -987,7 +1009,7 @@ int cs_mlp_set_params(cs_mlp *m, const float *host_in) {
     MLP_CUDA(m, cudaMemcpyAsync(m->master, host_in, kP * 4, cudaMemcpyHostToDevice, m->stream));
     MLP_CUDA(m, cudaMemsetAsync(m->m1, 0, kP * 4, m->stream));
     MLP_CUDA(m, cudaMemsetAsync(m->m2, 0, kP * 4, m->stream));
-    MLP_CUDA(m, cudaMemsetAsync(m->sse, 0, 16, m->stream));
+    MLP_CUDA(m, cudaMemsetAsync(m->failed, 0, sizeof(uint32_t), m->stream));
     int rc = refresh_copies(m);
     if (rc != CS_OK) return rc;
     MLP_CUDA(m, cudaStreamSynchronize(m->stream));
@@ -1021,7 +1043,7 @@ int cs_mlp_train_step(cs_mlp *m, int64_t n, const float *feat, const int32_t *ba
         return mfail(m, CS_ERR_ARG, "NULL or misaligned array");
     if (*m->gave_up()) return failed_step(m);
     MLP_CUDA(m, cudaSetDevice(m->device));
-    const int grid = grid_for(m, n, kTcGroups * kTcRows, 1);
+    const int grid = grid_for(m, n, kTcRows, 1);
     if (grid > m->n_part_cap) {
         MLP_CUDA(m, cudaStreamSynchronize(m->stream));
         cudaFree(m->partial);
@@ -1032,25 +1054,23 @@ int cs_mlp_train_step(cs_mlp *m, int64_t n, const float *feat, const int32_t *ba
     }
     const int tiles = (int)((n + kTcRows - 1) / kTcRows);
     Weights W{m->w1t, m->w2t, m->w2n, m->master};
-    uint32_t *err = reinterpret_cast<uint32_t *>(m->sse + 1);
     k_mlp_train<<<grid, kTcThreads, kSmemTc, m->stream>>>(n, tiles, feat, band, target, W, (float)(1.0 / (double)n),
-                                                          aligned(feat, 16), m->lose_product, m->partial, err,
+                                                          aligned(feat, 16), m->lose_product, m->partial, m->failed,
                                                           m->gave_up());
     MLP_CUDA(m, cudaGetLastError());
     const int64_t t = m->steps + 1;
     const float bc1 = (float)(1.0 - std::pow(0.9, (double)t)), bc2 = (float)(1.0 - std::pow(0.999, (double)t));
     k_mlp_adam<<<(kP + 1 + 31) / 32, 32 * kAdamWarps, 0, m->stream>>>(grid, m->partial, m->master, m->m1, m->m2, m->grad,
-                                                              m->w1t, m->w2t, m->w2n, lr, bc1, bc2, m->sse, err);
+                                                              m->w1t, m->w2t, m->w2n, lr, bc1, bc2, m->h_sse, m->failed);
     MLP_CUDA(m, cudaGetLastError());
     m->steps = t;
     if (loss_out) {
-        MLP_CUDA(m, cudaMemcpyAsync(m->h_sse, m->sse, 4, cudaMemcpyDeviceToHost, m->stream));
         MLP_CUDA(m, cudaStreamSynchronize(m->stream));
         if (*m->gave_up()) {
             m->steps = t - 1;
             return failed_step(m);
         }
-        *loss_out = (float)((double)m->h_sse[0] / (double)n);
+        *loss_out = (float)((double)*static_cast<volatile float *>(m->h_sse) / (double)n);
     }
     return CS_OK;
 }
