@@ -320,7 +320,10 @@ __device__ __noinline__ void settle_stop(Pixel &px, uint32_t g0, uint32_t g1, co
 
 // End of the group of pairs [g0, g1): T is T0 times the group's product
 // where that stays above the stop threshold, the pair-by-pair T (and where it
-// stopped) otherwise.
+// stopped) otherwise.  A pixel that is below the threshold by the product
+// alone stays open, but takes no more: its T is within 1,024 roundings (6e-5)
+// of the threshold, and every splat that counts takes at least 1/255 of it.
+// The chunks close such a pixel: the same image and list end.
 __device__ __forceinline__ void settle_group(Pixel &px, uint32_t g0, uint32_t g1, const uint32_t *__restrict__ pval,
                                              const float4 *__restrict__ rec) {
     const float Tq = px.T0 * px.P;

@@ -955,7 +955,10 @@ __global__ void __launch_bounds__(kProjThreads, 5) k_project(
 // transforms once for several chunks and launch fewer CTAs.
 // One chunk against eight: 16,384 Gaussians at 256x256 232 -> 218 us a frame,
 // 202,738 at 1280x720 405 -> 382 us, 100 x 12,661 509 -> 496 us (5,000
-// blocks); four against eight are equal from 16,384 blocks up.
+// blocks).  Four against one, frames of 3,176- and 65,536-Gaussian characters
+// at 1280x720: 1.4% slower at 3,000 blocks, equal within the runs' 0.5% from
+// 6,500 to 8,300, up to 1% faster from 9,000 to 16,000 (740 -> 736 us at
+// 9,000, 1,386 -> 1,371 at 12,000).
 constexpr int kProjChunks = 4;
 constexpr int kProjOneChunkBlocks = 8192;
 
